@@ -216,9 +216,13 @@ class UNet:
         c, shape = self.cache
         S = dY.shape[0]
         s1s, s2s, s3s = shape, half(shape), half(half(shape))
-        self.gW = {n: torch.zeros_like(w) for n, w in self.W32.items()}
+        # one zeroed allocation for all accumulators (a fill instead of 22)
+        params = [*self.W32.items(), *self.b32.items()]
+        parts = torch.zeros(self.n_params(), device=self.dev).split([p.numel() for _, p in params])
+        views = [z.view(p.shape) for z, (_, p) in zip(parts, params)]
+        self.gW = {n: z for n, z in zip(self.W32, views)}
         self.wgrad_inputs = {}
-        self.gb = {n: torch.zeros_like(b) for n, b in self.b32.items()}
+        self.gb = {n: z for n, z in zip(self.b32, views[len(self.W32):])}
         self._wgrad(c["u1"], dY, "out", S, s1s)
         d = self._conv_T(dY, "out", S, s1s)
         d = self._relu_bwd(d, c["u1"])
