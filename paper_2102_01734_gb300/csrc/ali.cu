@@ -12,6 +12,10 @@
 // of the stop test. Sweeps are launched back to back; each reads the
 // previous sweep's maxima and returns at once after the stop test is met,
 // so a fixed launch sequence serves any sweep count.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "rt3d_internal.cuh"
 
 namespace rt3d {
@@ -230,6 +234,246 @@ __global__ void __launch_bounds__(256) gs_colour_kernel(int nx, int ny, int nz, 
             jmax = fmax(jmax, fabs(nv));
         }
     }
+    block_max_atomic((double)dmax, &st->dmax[m]);
+    block_max_atomic((double)jmax, &st->jmax[m]);
+}
+
+// Half a sweep of the same iteration in one launch: the four colours of the
+// planes with parity pz, one cluster of blocks per plane. Planes of one parity
+// are no neighbours (z not periodic, or nz even), so their colours are ordered
+// by a barrier of the cluster instead of a launch. Each block owns `band` pairs
+// of rows and keeps the iterate of those rows, of the rows beside them and of
+// the planes above and below in shared memory, with a column beside either
+// edge: all 26 neighbours are read there without index arithmetic. A colour's
+// update goes to the copies beside the edges as well (in the neighbouring block
+// where the row beside is its own).
+// The next voxel's coefficients are loaded while a voxel is computed, across
+// the barriers too.
+// Sweep at 129^3 149 us with one launch per colour (gs_colour_kernel), 100 us
+// here; at 65^3 56 and 35 us. What bounds it is the latency of a voxel's
+// instructions at 16 warps per SM: a ring of coefficient blocks in shared memory
+// (cp.async) ran at 14 warps and 118 us, two smaller blocks per SM at 110 us.
+template <typename A> struct GsShared {
+    int pitch, rows;  // row pitch (nx + 2), rows of a plane (2 band + 2)
+    __host__ __device__ int plane() const { return rows * pitch; }
+    __host__ __device__ size_t bytes() const {
+        return (size_t)(3 * plane() + 2 * pitch + 2 * rows) * sizeof(A);
+    }
+};
+
+template <typename A, bool SEAM>
+__global__ void __launch_bounds__(512) gs_plane_kernel(int nx, int ny, int nz, ColourGeo cg, int pz,
+                                                       int band, GsShared<A> g, const A *__restrict__ a,
+                                                       const double *__restrict__ inv_diag,
+                                                       const double *__restrict__ r,
+                                                       const double *__restrict__ src,
+                                                       double *__restrict__ dst,
+                                                       const float *__restrict__ src32,
+                                                       float *__restrict__ dst32, int m, double tol,
+                                                       OsState *st, Periodic per) {
+    namespace coop = cooperative_groups;
+    constexpr bool f32 = sizeof(A) == 4;
+    if (st->done) return;
+    if (pz == 0 && m >= 2) {
+        const double dm = bitsd(st->dmax[m - 1]), jm = bitsd(st->jmax[m - 1]);
+        if (dm <= tol * jm) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                st->done = 1;
+                st->count = m - 1;
+            }
+            return;
+        }
+    }
+    coop::cluster_group cl = coop::this_cluster();
+    extern __shared__ __align__(16) unsigned char gs_smem[];
+    const int pitch = g.pitch;
+    A *const C = reinterpret_cast<A *>(gs_smem);  // this plane: rows y0 - 1 .. y1, columns -1 .. nx
+    const int L = g.plane(), H = 2 * L;  // below, above (all as offsets from C)
+    const int orow = 3 * L;              // last sweep's rows ny - 1 and 0 (an odd periodic y axis)
+    const int ocol = orow + 2 * pitch;   // last sweep's columns nx - 1 and 0 (an odd periodic x axis)
+    const int ranks = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int zi = blockIdx.x / ranks, z = 2 * zi + pz;
+    const int y0 = min(ny, 2 * band * rank), y1 = min(ny, y0 + 2 * band), h = y1 - y0;
+    const int nxy = nx * ny, vz = nxy * z;
+    const bool seamx = SEAM && per.x && (nx & 1), seamy = SEAM && per.y && (ny & 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // 1 / (voxels of a colour's row): the even columns, the odd ones. An index
+    // below 2^21 plus a half times it, truncated, is the quotient: the product is
+    // within 1.5e-4 of the quotient's value and the half keeps it 1 / (2 1024)
+    // away from the next integer.
+    const float inv0 = 1.0f / (float)((nx + 1) >> 1), inv1 = 1.0f / (float)max(1, nx >> 1);
+
+    // this block's voxels of colour q: indices [k0, k1) of the colour, its
+    // plane's first one at kz
+    auto range = [&](int q, int &kz, int &k0, int &k1) {
+        const int c = 4 * pz + q, nxc = cg.nxc[c], nyc = cg.nyc[c];
+        kz = nxc * nyc * zi;
+        k0 = kz + nxc * (y0 >> 1);
+        k1 = h > 0 ? kz + nxc * min((y1 - (q >> 1) + 1) >> 1, nyc) : k0;
+    };
+    // voxel (x, y) of index k
+    auto voxel = [&](int q, int k, int kz, int &x, int &y) {
+        const int nxc = (nx - (q & 1) + 1) >> 1;
+        const int yi = (int)(((float)(k - kz) + 0.5f) * (q & 1 ? inv1 : inv0));
+        x = 2 * (k - kz - yi * nxc) + (q & 1);
+        y = 2 * yi + (q >> 1);
+    };
+    struct Item {
+        A cf[26];
+        double rv, id;
+        int x, y;
+    };
+    auto load = [&](int q, int k, int kz, Item &w) {
+        const A *__restrict__ ab = a + os_colour_index(0, cg.blk[4 * pz + q], k);
+#pragma unroll
+        for (int p = 0; p < 26; ++p) w.cf[p] = ab[p * 32];
+        voxel(q, k, kz, w.x, w.y);
+        const int gv = w.x + nx * w.y + vz;
+        w.rv = r[gv];
+        w.id = inv_diag[gv];
+    };
+    int kz, first, end;
+    range(0, kz, first, end);
+    int k = first + threadIdx.x;
+    bool ok = k < end;
+    Item w;
+    if (ok) load(0, k, kz, w);
+
+    // the rows: last sweep's values of this plane; of the planes below and
+    // above last sweep's for the even planes, this sweep's for the odd ones (a
+    // clamped plane, with zero coefficients, is the voxel's own)
+    const A *__restrict__ old, *__restrict__ now;
+    if constexpr (f32) {
+        old = src32;
+        now = dst32;
+    } else {
+        old = src;
+        now = dst;
+    }
+    const A *plane = old + vz;
+    const int zl = os_nb_lo(z, nz, per.z), zh = os_nb_hi(z, nz, per.z);
+    const A *below = (zl == z || pz == 0 ? old : now) + (long long)nxy * zl;
+    const A *above = (zh == z || pz == 0 ? old : now) + (long long)nxy * zh;
+    auto edge_x = [&](int xx) {  // the voxel behind column xx of a row
+        const int x = xx - 1;
+        return x < 0 ? (per.x ? nx - 1 : 0) : (x >= nx ? (per.x ? 0 : nx - 1) : x);
+    };
+    for (int i = warp; i < (h > 0 ? 3 * (h + 2) : 0); i += (int)(blockDim.x >> 5)) {
+        const int p = i / (h + 2), ys = i - p * (h + 2);
+        int y = y0 + ys - 1;
+        if (y < 0) y = per.y ? ny - 1 : 0;
+        if (y >= ny) y = per.y ? 0 : ny - 1;
+        const A *from = (p == 0 ? plane : (p == 1 ? below : above)) + y * nx;
+        A *to = C + p * g.plane() + ys * pitch;
+        for (int xx = lane; xx < pitch; xx += 32) to[xx] = from[edge_x(xx)];
+    }
+    if (seamy)
+        for (int i = threadIdx.x; i < 2 * pitch; i += blockDim.x) {
+            const int k = i >= pitch;
+            C[orow + i] = plane[edge_x(i - k * pitch) + (k ? 0 : nx * (ny - 1))];
+        }
+    if (seamx)
+        for (int i = threadIdx.x; i < 2 * h; i += blockDim.x) {
+            const int k = i >= h, ys = i - k * h;
+            C[ocol + k * g.rows + ys + 1] = plane[(k ? 0 : nx - 1) + nx * (y0 + ys)];
+        }
+    // the copies of this block's first and last row beside other blocks' rows
+    // (or its own, where the plane wraps onto the same block)
+    const int last = (ny - 1) / (2 * band);  // the rank that owns the last row
+    A *lo = nullptr, *hi = nullptr;
+    if (h > 0) {
+        if (y0 > 0) lo = cl.map_shared_rank(C, rank - 1) + (2 * band + 1) * pitch;
+        else if (per.y) lo = cl.map_shared_rank(C, last) + (ny - 2 * band * last + 1) * pitch;
+        if (y1 < ny) hi = cl.map_shared_rank(C, rank + 1);
+        else if (per.y) hi = cl.map_shared_rank(C, 0);
+    }
+    cl.sync();
+    A dmax = A(0), jmax = A(0);
+    // results are stored one voxel later: a barrier waits for the block's
+    // stores, and those of its last voxels would be on their way still
+    double pv = 0.0;
+    int pg = -1;
+    auto store = [&]() {
+        if (pg < 0) return;
+        dst[pg] = pv;
+        if constexpr (f32) dst32[pg] = (float)pv;
+        pg = -1;
+    };
+    for (int q = 0, left = -1;;) {
+        if (left < 0) left = max(1, (end - first + (int)blockDim.x - 1) / (int)blockDim.x);
+        k += blockDim.x;
+        int nq = q;
+        if (left == 1 && q < 3) {
+            range(++nq, kz, first, end);
+            k = first + (int)threadIdx.x;
+        }
+        const bool nok = k < end;
+        Item nw;
+        if (nok) load(nq, k, kz, nw);
+        store();
+        if (ok) {
+            const int x = w.x, y = w.y;
+            const int ys = y - y0 + 1, at = ys * pitch + x;
+            const bool ex[3] = {seamx && x == 0, true, seamx && x == nx - 1};
+            const bool ey[3] = {seamy && y == 0, true, seamy && y == ny - 1};
+            A acc = A(0);
+#pragma unroll
+            for (int d = 0, p = 0; d < 27; ++d) {
+                if (d == 13) continue;
+                const int i = d % 3, j = (d / 3) % 3, o = at + (j - 1) * pitch + i;
+                A xv;
+                if (d < 9) xv = C[L + o];
+                else if (d >= 18) xv = C[H + o];
+                else if (!SEAM) xv = C[o];
+                else {
+                    // a neighbour of the same colour (across the seam of an
+                    // odd periodic axis): its value of the last sweep
+                    const int u = j == 1 ? ocol + (i == 2 ? g.rows : 0) + ys
+                                         : orow + (j == 2 ? pitch : 0) + x + i;
+                    xv = C[ex[i] && ey[j] ? u : o];
+                }
+                acc += w.cf[p] * xv;
+                ++p;
+            }
+            const double nv = (w.rv + (double)acc) * w.id;
+            pv = nv;
+            pg = x + nx * y + vz;
+            A val;
+            const A was = C[at + 1];
+            if constexpr (f32) {
+                val = (float)nv;
+                dmax = fmaxf(dmax, fabsf(val - was));
+                jmax = fmaxf(jmax, fabsf(val));
+            } else {
+                val = nv;
+                dmax = fmax(dmax, fabs(val - was));
+                jmax = fmax(jmax, fabs(val));
+            }
+            if (q < 3) {
+                C[at + 1] = val;
+                const bool row = y == y0 || y == y1 - 1, col = per.x && (x == 0 || x == nx - 1);
+                if (row || col) {
+                    const int e = x == 0 ? nx + 1 : 0;
+                    if (col) C[ys * pitch + e] = val;
+                    if (lo && y == y0) {
+                        lo[x + 1] = val;
+                        if (col) lo[e] = val;
+                    }
+                    if (hi && y == y1 - 1) {
+                        hi[x + 1] = val;
+                        if (col) hi[e] = val;
+                    }
+                }
+            }
+        }
+        ok = nok;
+        w = nw;
+        if (--left > 0) continue;
+        if (q++ == 3) break;
+        cl.sync();
+        left = -1;
+    }
+    store();
     block_max_atomic((double)dmax, &st->dmax[m]);
     block_max_atomic((double)jmax, &st->jmax[m]);
 }
@@ -560,10 +804,77 @@ ColourGeo colour_geo(int nx, int ny, int nz) {
     return cg;
 }
 
+// Blocks per plane and pairs of rows per block of the plane kernel: the
+// smallest cluster that fits its rows into shared memory and gives the GPU a
+// block per SM from the planes of one parity, at most 8. False where the
+// kernel does not apply: the planes of one parity meet across a periodic z
+// axis of odd length, or a plane's rows do not fit.
+template <typename A>
+static bool gs_plane_shape(int nx, int ny, int nz, Periodic per, int *ranks, int *band,
+                           GsShared<A> *g) {
+    if (per.z && (nz & 1)) return false;
+    const int pairs = (ny + 1) / 2, planes = (nz + 1) / 2;
+    for (*ranks = 1; *ranks <= 8; *ranks *= 2) {
+        *band = (pairs + *ranks - 1) / *ranks;
+        *g = GsShared<A>{nx + 2, 2 * *band + 2};
+        const bool full = (long long)planes * *ranks * 4 >= 3LL * device_sm_count();
+        if (g->bytes() <= 220 * 1024 && (full || *ranks == 8 || *band == 1)) return true;
+    }
+    return false;
+}
+
+template <typename A, bool SEAM>
+static cudaError_t gs_planes(int nx, int ny, int nz, const ColourGeo &cg, int ranks, int band,
+                             const GsShared<A> &g, const A *a, const double *inv_diag, const double *r,
+                             const double *src, double *dst, const float *src32, float *dst32, int m,
+                             double tol, OsState *st, cudaStream_t s, Periodic per) {
+    const size_t shm = g.bytes();
+    if (shm > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            gs_plane_kernel<A, SEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ranks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
+    lc.blockDim = dim3(std::min(512, (band * ((nx + 1) / 2) + 31) / 32 * 32));
+    lc.dynamicSmemBytes = shm;
+    lc.stream = s;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    for (int pz = 0; pz < 2 && pz < nz; ++pz) {
+        lc.gridDim = dim3((nz - pz + 1) / 2 * ranks);
+        const cudaError_t e =
+            cudaLaunchKernelEx(&lc, gs_plane_kernel<A, SEAM>, nx, ny, nz, cg, pz, band, g, a, inv_diag, r,
+                               src, dst, src32, dst32, m, tol, st, per);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_gs_sweep(int nx, int ny, int nz, const ColourGeo &cg, const void *a, bool a64,
                             const double *inv_diag, const double *r, const double *src,
                             double *dst, const float *src32, float *dst32, int m, double tol,
-                            OsState *st, cudaStream_t s, Periodic per) {
+                            OsState *st, cudaStream_t s, Periodic per, int *launches) {
+    cudaError_t e = cudaSuccess;
+    auto planes = [&](auto coef, const auto *x) -> bool {
+        using A = decltype(coef);
+        int ranks = 0, band = 0;
+        GsShared<A> g{};
+        if (!gs_plane_shape<A>(nx, ny, nz, per, &ranks, &band, &g)) return false;
+        *launches = nz > 1 ? 2 : 1;
+        const bool seam = (per.x && (nx & 1)) || (per.y && (ny & 1));
+        e = seam ? gs_planes<A, true>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
+                                      dst32, m, tol, st, s, per)
+                 : gs_planes<A, false>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
+                                       dst32, m, tol, st, s, per);
+        return true;
+    };
+    if (a64 ? planes(0.0, static_cast<const double *>(a)) : planes(0.0f, static_cast<const float *>(a)))
+        return e;
+    *launches = 8;
     for (int c = 0; c < 8; ++c) {
         const int blocks = grid_for(cg.cnt[c] > 0 ? cg.cnt[c] : 1, 256);
         if (a64)

@@ -628,15 +628,16 @@ rt3d_status os_solve_dev(rt3d_grid *g, const double *Jfs, const double *J, const
         return RT3D_OK;
     }
     if (g->os_kind == kOsGaussSeidel) {
-        // eight launches per sweep; the stop flag is read every fourth sweep
+        // the stop flag is read every fourth sweep
+        int launches = 0;
         const ColourGeo cg = colour_geo(g->nx, g->ny, g->nz);
         for (int m = 1; m <= max_sweeps; ++m) {
             CK(launch_gs_sweep(g->nx, g->ny, g->nz, cg, g->a, g->a64, g->inv_diag, g->r,
                                g->dJ[(m - 1) & 1], g->dJ[m & 1],
                                g->a64 ? nullptr : g->dJ32[(m - 1) & 1],
                                g->a64 ? nullptr : g->dJ32[m & 1], m, tol, g->st, g->stream,
-                               g->per));
-            g->launches += 8;
+                               g->per, &launches));
+            g->launches += launches;
             if ((m & 3) == 0 && m < max_sweeps) {
                 int done = 0;
                 CK(cudaMemcpyAsync(&done, &g->st->done, sizeof done, cudaMemcpyDeviceToHost,

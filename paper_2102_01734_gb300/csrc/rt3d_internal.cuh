@@ -272,11 +272,12 @@ cudaError_t launch_os_prep(int nx, int ny, int nz, const double *lstar, const do
 // for colour 0 .. 7, every voxel of the colour from the neighbours' values
 // of this sweep (earlier colours, in dst) or of the last (src); the stop test
 // of sweep m - 1 first (as launch_os_sweep).
-// src32/dst32: FP32 copies of src/dst (mixed mode; unused with a64)
+// src32/dst32: FP32 copies of src/dst (mixed mode; unused with a64). *launches:
+// kernels launched.
 cudaError_t launch_gs_sweep(int nx, int ny, int nz, const ColourGeo &cg, const void *a, bool a64,
                             const double *inv_diag, const double *r, const double *src,
                             double *dst, const float *src32, float *dst32, int m, double tol,
-                            OsState *st, cudaStream_t s, Periodic per);
+                            OsState *st, cudaStream_t s, Periodic per, int *launches);
 // BiCGStab on [1 - Lambda*(1 - eps)] x = r from x = 0 (van der Vorst):
 // device scalars and the kernels of one iteration.
 struct BicgState {

@@ -1,0 +1,41 @@
+"""The Gauss-Seidel plane kernel where its split changes: one block to eight
+per plane, blocks without rows, odd and even axes, one layer, both precisions,
+and the spherical grid's axes (phi periodic, odd and even)."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [(4, 4, 1), (5, 4, 2), (6, 37, 3), (9, 16, 5), (33, 70, 9), (4, 6, 130),
+                               (130, 5, 260), (64, 10, 33)])
+@pytest.mark.parametrize("fp64", [True, False])
+def test_against_oracle(n, fp64):
+    from paper_2102_01734_gb300 import rt3d
+
+    nx, ny, nz = n
+    rng = np.random.default_rng(nx + ny + nz)
+    N = nx * ny * nz
+    L = rng.uniform(0.0, 1.0, (N, 27))
+    L *= 0.9 / L.sum(1, keepdims=True)
+    z = np.arange(N) // (nx * ny)
+    L[z == 0, :9] = 0.0
+    L[z == nz - 1, 18:] = 0.0
+    eps = 10.0 ** rng.uniform(-4, -1, (nz, ny, nx))
+    r = rng.standard_normal((nz, ny, nx))
+    g = rt3d.Grid(n, 2, 4, rt3d.LINEAR, rt3d.FP64 if fp64 else rt3d.FP32_FS_FP64_ALI)
+    g.set_os_solver(rt3d.OS_GAUSS_SEIDEL)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda")
+    for sweeps in (1, 6):
+        ref, m = oracle.os_gauss_seidel(L, eps, r, sweeps, 1e-14, colored=True)
+        x, k = g.os_solve(d(L.T), d(eps), d(r), max_sweeps=sweeps, tol=1e-14)
+        x = x.cpu().numpy()
+        assert k == m == sweeps
+        # FP32 mode: coefficients and neighbours rounded to 2^-24; the rows sum
+        # to at most 0.9, so sweeps damp the errors they inherit
+        tol = 1e-13 if fp64 else 2 * 27 * 2.0 ** -24 / (1 - 0.9)
+        assert np.max(np.abs(x - ref.reshape(x.shape))) <= tol * np.max(np.abs(ref))
+    g.close()
