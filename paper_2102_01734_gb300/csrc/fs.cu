@@ -644,6 +644,8 @@ __global__ void pair_pack_kernel(int nx, int ny, int nz, const float2 *__restric
 // one FMA between.
 template <bool PARAB>
 __global__ void __launch_bounds__(128) fs64_fast_kernel(FsParams p) {
+    __shared__ double tab[64];
+    exp_table(tab);
     const int nray = p.nx * p.ny;
     const int ray = blockIdx.x * blockDim.x + threadIdx.x;
     if (ray >= nray) return;
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(128) fs64_fast_kernel(FsParams p) {
         const double hn = cn.x * rn.x;
         const double dSn = cn.y - Sc;
         const double w = hc + hn;
-        const IntervalDE f = interval64<PARAB>(u, ru);
+        const IntervalDE f = interval64<PARAB>(u, ru, tab);
         // difference form of the update (as in the FP32 kernel)
         double In = fma(f.e0, Sp - I, I);
         In = fma(f.a, dS, In);
@@ -702,7 +704,7 @@ __global__ void __launch_bounds__(128) fs64_fast_kernel(FsParams p) {
         vc = vn;
         cwc = rn.y;
     }
-    const IntervalDE f = interval64<PARAB>(u, ru);
+    const IntervalDE f = interval64<PARAB>(u, ru, tab);
     I = fma(f.a, dS, fma(f.e0, Sp - I, I));
     atomicAdd(J + vc, cwc * I);
 }

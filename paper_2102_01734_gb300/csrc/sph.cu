@@ -666,6 +666,8 @@ __global__ void __launch_bounds__(128) sph_fs_fast_kernel(SphFsParams p, double 
 // at the replicated index (folded afterwards).
 template <bool PARAB>
 __global__ void __launch_bounds__(128) sph_fs64_fast_kernel(SphFsParams p, double *__restrict__ Jrep) {
+    __shared__ double tab[64];
+    exp_table(tab);
     const long long ray = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (ray >= p.nrays) return;
     const long long s0 = p.ray_off[ray];
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(128) sph_fs64_fast_kernel(SphFsParams p, doubl
         const double hn = cn.x * (0.5 * __ldg(l64 + k));
         const double dSn = cn.y - Sc;
         const double w = hc + hn;
-        const IntervalDE f = interval64<PARAB>(u, ru);
+        const IntervalDE f = interval64<PARAB>(u, ru, tab);
         double In = fma(f.e0, Sp - I, I);
         In = fma(f.a, dS, In);
         if (PARAB) {
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(128) sph_fs64_fast_kernel(SphFsParams p, doubl
         vc = vn;
         cwc = (double)r.y + (double)r.w;
     }
-    const IntervalDE f = interval64<PARAB>(u, ru);
+    const IntervalDE f = interval64<PARAB>(u, ru, tab);
     I = fma(f.a, dS, fma(f.e0, Sp - I, I));
     atomicAdd(Jrep + vc, cwc * I);
 }
