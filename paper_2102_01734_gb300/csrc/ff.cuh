@@ -48,6 +48,13 @@ __device__ __forceinline__ ff ff_add(ff x, ff y) {
 
 __device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
 
+// x + y and x - y for |x| >= |y| (three operations fewer)
+__device__ __forceinline__ ff ff_add_big(ff x, ff y) {
+    const ff s = quick_two_sum(x.hi, y.hi);
+    return quick_two_sum(s.hi, s.lo + (x.lo + y.lo));
+}
+__device__ __forceinline__ ff ff_sub_big(ff x, ff y) { return ff_add_big(x, ff_neg(y)); }
+
 __device__ __forceinline__ ff ff_add_f(ff x, float y) {
     const ff s = two_sum(x.hi, y);
     return quick_two_sum(s.hi, s.lo + x.lo);
@@ -63,6 +70,26 @@ __device__ __forceinline__ ff ff_mul_f(ff x, float y) {
     return quick_two_sum(p.hi, fmaf(x.lo, y, p.lo));
 }
 
+// x * y without the last renormalisation: the same sum, its low part up to an
+// ulp of the high one. As a factor or an addend of a further operation, which
+// drops only lo * lo (2^-46 of the product at most).
+__device__ __forceinline__ ff ff_mul_raw(ff x, ff y) {
+    const ff p = two_prod(x.hi, y.hi);
+    return ff{p.hi, fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, p.lo))};
+}
+
+// x * y + z for |z| >= |x y|; the same without the last renormalisation
+__device__ __forceinline__ ff ff_fma_big_raw(ff x, ff y, ff z) {
+    const ff p = two_prod(x.hi, y.hi);
+    const float e = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, p.lo));
+    const ff s = quick_two_sum(z.hi, p.hi);
+    return ff{s.hi, s.lo + (e + z.lo)};
+}
+__device__ __forceinline__ ff ff_fma_big(ff x, ff y, ff z) {
+    const ff s = ff_fma_big_raw(x, y, z);
+    return quick_two_sum(s.hi, s.lo);
+}
+
 // x * y + z
 __device__ __forceinline__ ff ff_fma(ff x, ff y, ff z) {
     const ff p = two_prod(x.hi, y.hi);
@@ -74,14 +101,16 @@ __device__ __forceinline__ ff ff_fma(ff x, ff y, ff z) {
 // exact scaling by a power of two (no overflow or underflow in range)
 __device__ __forceinline__ ff ff_scale(ff x, float p2) { return ff{x.hi * p2, x.lo * p2}; }
 
-// 1/x for x > 0: FP32 reciprocal r, then one Newton-Raphson step
-// r + r (1 - x r) with the residual 1 - x r formed exactly enough in
-// float-float (it is ~2^-23, so its FP32 product with r adds < 2^-46).
+// 1/x for x > 0: r the FP32 approximation (relative error e <= 2^-23), then
+// r (1 + e + e^2) with e = 1 - x r formed by two fused operations (it is exact
+// to 2^-24 of itself, as the product with r is): 2^-47 in all, and nine
+// instructions where a float-float residual and a correctly rounded r took
+// about 28 for the same accuracy.
 __device__ __forceinline__ ff ff_recip(ff x) {
-    const float r = __frcp_rn(x.hi);
-    const ff xr = ff_mul_f(x, r);
-    const ff e = ff_sub(ff_of(1.0f), xr);
-    return quick_two_sum(r, r * e.hi);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x.hi));
+    const float e = fmaf(-x.lo, r, fmaf(-x.hi, r, 1.0f));
+    return quick_two_sum(r, r * fmaf(e, e, e));
 }
 
 // FP64 value of a float-float (the widening of each part is exact; the sum

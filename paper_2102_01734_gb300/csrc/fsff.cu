@@ -39,7 +39,8 @@ __device__ __forceinline__ ff ff_exp_neg(ff u, const float2 *tab) {
     ff r = two_sum(fmaf(-nf, kC1, u.hi), -nf * kC2);
     r = ff_add_f(r, u.lo);
     r = ff_sub(r, ff_mul_f(ff{kC3, kC4}, nf));
-    ff e = ff_add(ff_sub(ff_of(1.0f), r), ff_scale(ff_mul(r, r), 0.5f));
+    // |r| < 1/46, r^2/2 < 1 - r
+    ff e = ff_add_big(ff_sub_big(ff_of(1.0f), r), ff_scale(ff_mul_raw(r, r), 0.5f));
     const float x = r.hi;
     e = ff_add_f(e, x * x * x * fmaf(x, fmaf(-x, 1.0f / 120.0f, 1.0f / 24.0f), -1.0f / 6.0f));
     const float2 t = tab[n & 31];
@@ -65,21 +66,23 @@ __device__ __forceinline__ IntervalFF interval_ff(ff u, ff ru, const float2 *tab
         q = fmaf(q, u.hi, 4.935483e-08f);
         q = fmaf(q, u.hi, -5.5071155e-07f);
         q = fmaf(q, u.hi, 5.51131e-06f);
-        ff P = ff_fma(ff_of(q), u, ff{-4.9603143e-05f, 1.6644579e-12f});
-        P = ff_fma(P, u, ff{3.968254e-04f, -9.971136e-12f});
-        P = ff_fma(P, u, ff{-2.7777778e-03f, 6.7610896e-11f});
-        P = ff_fma(P, u, ff{1.6666668e-02f, -8.692481e-10f});
-        P = ff_fma(P, u, ff{-8.3333336e-02f, 2.4835272e-09f});
-        P = ff_fma(P, u, ff{3.3333334e-01f, -9.934108e-09f});
+        // every constant exceeds the term added to it (ratios below 1/8), which
+        // the renormalisation left out is damped by as well
+        ff P = ff_fma_big_raw(ff_of(q), u, ff{-4.9603143e-05f, 1.6644579e-12f});
+        P = ff_fma_big_raw(P, u, ff{3.968254e-04f, -9.971136e-12f});
+        P = ff_fma_big_raw(P, u, ff{-2.7777778e-03f, 6.7610896e-11f});
+        P = ff_fma_big_raw(P, u, ff{1.6666668e-02f, -8.692481e-10f});
+        P = ff_fma_big_raw(P, u, ff{-8.3333336e-02f, 2.4835272e-09f});
+        P = ff_fma_big(P, u, ff{3.3333334e-01f, -9.934108e-09f});
         const ff b = ff_mul(u, P);
         const ff hu = ff_scale(u, 0.5f);
-        r.a = ff_sub(hu, ff_mul(hu, b));
-        r.e0 = ff_sub(u, ff_mul(u, r.a));
-        r.d = ff_sub(r.a, b);
+        r.a = ff_fma_big(ff_neg(hu), b, hu);    // b < 1/6
+        r.e0 = ff_fma_big(ff_neg(u), r.a, u);   // a < 1/4
+        r.d = ff_sub_big(r.a, b);               // b < u/3 < a
     } else {
-        r.e0 = ff_sub(ff_of(1.0f), ff_exp_neg(u, tab));
-        r.a = ff_sub(ff_of(1.0f), ff_mul(r.e0, ru));
-        r.d = ff_mul(ff_sub(ff_scale(r.a, 2.0f), r.e0), ru);
+        r.e0 = ff_sub_big(ff_of(1.0f), ff_exp_neg(u, tab));
+        r.a = ff_fma_big(ff_neg(r.e0), ru, ff_of(1.0f));
+        r.d = ff_mul(ff_sub_big(ff_scale(r.a, 2.0f), r.e0), ru);  // a > e0/2
     }
     return r;
 }
@@ -122,11 +125,9 @@ __device__ __forceinline__ void ff_advance(RayFF &s, ff hn, ff Sn, const float2 
     if (PARAB) {
         const ff q = ff_mul(s.u, rw);
         if (s.u.hi < 1.0f && q.hi < 4.0f) {
-            ff fw = ff_of(1.0f);
-            if (!(s.u.hi < 0.5f)) fw = ff_sub(ff_of(2.0f), ff_scale(s.u, 2.0f));
-            if (!(q.hi < 2.0f)) fw = ff_mul(fw, ff_sub(ff_of(2.0f), ff_scale(q, 0.5f)));
-            const ff sr = ff_mul(s.u, ff_recip_floor(ff_add(s.u, w)));
-            const ff sd = ff_mul(ff_mul(fw, sr), f.d);
+            ff sd = ff_mul(ff_mul_raw(s.u, ff_recip_floor(ff_add(s.u, w))), f.d);
+            if (!(s.u.hi < 0.5f)) sd = ff_mul(sd, ff_sub_big(ff_of(2.0f), ff_scale(s.u, 2.0f)));
+            if (!(q.hi < 2.0f)) sd = ff_mul(sd, ff_sub_big(ff_of(2.0f), ff_scale(q, 0.5f)));
             In = ff_fma(sd, ff_fma(ff_neg(q), dSn, s.dS), In);
         }
     }
@@ -189,13 +190,13 @@ __global__ void __launch_bounds__(128) fsff_kernel(FsParams p, const float4 *__r
         const float4 rn = __ldg(rf + k);
         const float4 cn = chiS[vn];
         ff_advance<PARAB>(st, ff_mul(ff{cn.x, cn.y}, ff{rn.x, rn.y}), ff{cn.z, cn.w}, tab);
-        const ff c = ff_mul(cw, st.I);
+        const ff c = ff_mul_raw(cw, st.I);
         atomicAdd(J + vc, widen_f32(c.hi) + widen_f32(c.lo));
         vc = vn;
         cw = ff{rn.z, rn.w};
     }
     ff_last(st, tab);
-    const ff c = ff_mul(cw, st.I);
+    const ff c = ff_mul_raw(cw, st.I);
     atomicAdd(J + vc, widen_f32(c.hi) + widen_f32(c.lo));
     if (!(fabsf(st.I.hi) <= 3.402823466e38f))  // non-finite: make J NaN
         atomicAdd(J + vc, __longlong_as_double(0x7ff8000000000000LL));
@@ -244,13 +245,13 @@ __global__ void __launch_bounds__(128) sph_fsff_kernel(SphFsParams p, const floa
         const float4 cn = chiS[vn];
         ff_advance<PARAB>(st, ff_mul(ff{cn.x, cn.y}, half_chord_ff(r.z, __ldg(l64 + k))),
                           ff{cn.z, cn.w}, tab);
-        const ff c = ff_mul(cw, st.I);
+        const ff c = ff_mul_raw(cw, st.I);
         atomicAdd(Jrep + vc, widen_f32(c.hi) + widen_f32(c.lo));
         vc = vn;
         cw = ff{r.y, r.w};
     }
     ff_last(st, tab);
-    const ff c = ff_mul(cw, st.I);
+    const ff c = ff_mul_raw(cw, st.I);
     atomicAdd(Jrep + vc, widen_f32(c.hi) + widen_f32(c.lo));
     if (!(fabsf(st.I.hi) <= 3.402823466e38f))  // non-finite: make J NaN
         atomicAdd(Jrep + vc, __longlong_as_double(0x7ff8000000000000LL));
