@@ -619,6 +619,17 @@ rt3d_status os_solve_dev(rt3d_grid *g, const double *Jfs, const double *J, const
     CK(launch_os_init((int)g->N, Jfs, J, extra, g->inv_diag, g->r, g->dJ[0],
                       g->a64 ? nullptr : g->dJ32[0], g->st, g->stream));
     ++g->launches;
+    if (g->os_kind != kOsBicgstab) {
+        bool ran = false;
+        CK(launch_os_resident(g->nx, g->ny, g->nz, g->os_kind == kOsGaussSeidel, g->a, g->a64,
+                              g->inv_diag, g->r, g->dJ, g->a64 ? nullptr : g->dJ32, max_sweeps, tol,
+                              g->st, g->stream, g->per, &ran));
+        if (ran) {
+            CK(launch_os_finish(max_sweeps, tol, g->st, g->stream));
+            g->launches += 2;
+            return RT3D_OK;
+        }
+    }
     if (g->os_kind == kOsJacobi) {
         for (int m = 1; m <= max_sweeps; ++m)
             CK(launch_os_sweep(g->nx, g->ny, g->nz, g->a, g->a64, g->inv_diag, g->r, g->dJ,

@@ -304,6 +304,13 @@ cudaError_t launch_os_sweep(int nx, int ny, int nz, const void *a, bool a64,
                             const double *inv_diag, const double *r, double *const *buf,
                             float *const *buf32, int m, double tol, OsState *st, cudaStream_t s,
                             Periodic per = {true, true, false});
+// All sweeps 1 .. max_sweeps (Jacobi, or eight-colour Gauss-Seidel with gs) of
+// a small grid in one launch; *ran: whether the grid is small enough (nothing
+// launched otherwise). launch_os_finish follows as after single sweeps.
+cudaError_t launch_os_resident(int nx, int ny, int nz, bool gs, const void *a, bool a64,
+                               const double *inv_diag, const double *r, double *const *buf,
+                               float *const *buf32, int max_sweeps, double tol, OsState *st,
+                               cudaStream_t s, Periodic per, bool *ran);
 cudaError_t launch_os_finish(int max_sweeps, double tol, OsState *st, cudaStream_t s);
 cudaError_t launch_ali_update(int n, double *J, double *const *buf, OsState *st,
                               double *dJ_out, cudaStream_t s);
