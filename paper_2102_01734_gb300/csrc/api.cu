@@ -1327,7 +1327,7 @@ rt3d_status krylov_setup(rt3d_grid *g) {
     TRY(g->alloc(&g->dV, m + 1));
     TRY(g->alloc(&g->dZ, m));
     TRY(g->alloc(&g->dOne, 1));
-    TRY(g->alloc(&g->dots, m + 1));
+    TRY(g->alloc(&g->dots, 2 * m + 1));  // orthogonalise: two sets and a norm
     TRY(g->alloc(&g->coef, m + 1));
     CK(cudaMemcpyAsync(g->dV, g->V, sizeof(double *) * (m + 1), cudaMemcpyHostToDevice, g->stream));
     CK(cudaMemcpyAsync(g->dZ, g->Z, sizeof(double *) * m, cudaMemcpyHostToDevice, g->stream));
@@ -1350,6 +1350,29 @@ rt3d_status knorm(rt3d_grid *g, const double *w, double *out) {
     double d = 0.0;
     TRY(kdots(g, g->dOne, 1, w, &d));
     *out = std::sqrt(std::max(d, 0.0));
+    return RT3D_OK;
+}
+
+// Classical Gram-Schmidt, twice, of V[k] against V[0 .. k-1], then V[k] /=
+// |V[k]|: h[i] the summed coefficients, *hn the norm. The coefficients stay on
+// the device between the kernels; the host waits once.
+rt3d_status orthogonalise(rt3d_grid *g, int k, double *h, double *hn) {
+    const int n = (int)g->N;
+    double *const w = g->V[k], *const d1 = g->dots, *const d2 = d1 + k, *const d3 = d2 + k;
+    CK(cudaMemsetAsync(d1, 0, sizeof(double) * (2 * k + 1), g->stream));
+    CKL(launch_multi_dot(n, g->dV, k, w, d1, g->stream));
+    CKL(launch_multi_axpy(n, w, g->dV, d1, k, g->stream));
+    CKL(launch_multi_dot(n, g->dV, k, w, d2, g->stream));
+    CKL(launch_multi_axpy(n, w, g->dV, d2, k, g->stream));
+    CKL(launch_multi_dot(n, g->dV + k, 1, w, d3, g->stream));
+    CKL(launch_normalise(n, w, d3, w, g->stream));
+    std::vector<double> host(2 * k + 1);
+    CK(cudaMemcpyAsync(host.data(), d1, sizeof(double) * (2 * k + 1), cudaMemcpyDeviceToHost,
+                       g->stream));
+    CK(cudaStreamSynchronize(g->stream));
+    for (int i = 0; i < k; ++i) h[i] = host[i] + host[k + i];
+    *hn = std::sqrt(std::max(host[2 * k], 0.0));
+    if (!(host[2 * k] == host[2 * k])) *hn = host[2 * k];
     return RT3D_OK;
 }
 
@@ -1405,22 +1428,15 @@ rt3d_status fgmres(rt3d_grid *g, const FsParams &fphom, bool fp64, const double 
     if (!(beta > 0.0)) return RT3D_OK;
     if (!std::isfinite(beta)) return fail(RT3D_ENUMERIC, "non-finite residual norm");
     CKL(launch_scale_copy(n, r, 1.0 / beta, g->V[0], g->stream));
-    std::vector<double> H((m + 1) * m, 0.0), cs(m, 0.0), sn(m, 0.0), gv(m + 1, 0.0), h(m + 1),
-        h2(m + 1);
+    std::vector<double> H((m + 1) * m, 0.0), cs(m, 0.0), sn(m, 0.0), gv(m + 1, 0.0), h(m + 1);
     gv[0] = beta;
     int k = 0;
     for (int j = 0; j < m; ++j) {
         TRY(precond(g, g->V[j], g->Z[j]));
         TRY(apply_A(g, fphom, fp64, g->Z[j], g->V[j + 1]));
-        TRY(kdots(g, g->dV, j + 1, g->V[j + 1], h.data()));
-        TRY(kaxpy(g, g->V[j + 1], g->dV, h.data(), j + 1));
-        TRY(kdots(g, g->dV, j + 1, g->V[j + 1], h2.data()));
-        TRY(kaxpy(g, g->V[j + 1], g->dV, h2.data(), j + 1));
-        for (int i = 0; i <= j; ++i) h[i] += h2[i];
         double hn = 0.0;
-        TRY(knorm(g, g->V[j + 1], &hn));
+        TRY(orthogonalise(g, j + 1, h.data(), &hn));
         if (!std::isfinite(hn)) return fail(RT3D_ENUMERIC, "non-finite Krylov vector");
-        if (hn > 0.0) CKL(launch_scale_copy(n, g->V[j + 1], 1.0 / hn, g->V[j + 1], g->stream));
         // Givens rotations on column j
         for (int i = 0; i < j; ++i) {
             const double a = h[i], b = h[i + 1];

@@ -51,6 +51,13 @@ __global__ void scale_copy_kernel(int n, const double *src, double alpha, double
         dst[i] = alpha * src[i];
 }
 
+// dst = src / sqrt(*norm2)
+__global__ void normalise_kernel(int n, const double *src, const double *norm2, double *dst) {
+    const double alpha = 1.0 / sqrt(*norm2);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        dst[i] = alpha * src[i];
+}
+
 __global__ void sub_kernel(int n, const double *a, const double *b, double *out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         out[i] = a[i] - b[i];
@@ -78,6 +85,12 @@ cudaError_t launch_multi_axpy(int n, double *w, const double *const *V, const do
 
 cudaError_t launch_scale_copy(int n, const double *src, double alpha, double *dst, cudaStream_t s) {
     scale_copy_kernel<<<blocks_for(n, 256, 8 * device_sm_count()), 256, 0, s>>>(n, src, alpha, dst);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_normalise(int n, const double *src, const double *norm2, double *dst,
+                             cudaStream_t s) {
+    normalise_kernel<<<blocks_for(n, 256, 8 * device_sm_count()), 256, 0, s>>>(n, src, norm2, dst);
     return cudaGetLastError();
 }
 

@@ -453,6 +453,9 @@ cudaError_t launch_multi_dot(int n, const double *const *V, int k, const double 
 cudaError_t launch_multi_axpy(int n, double *w, const double *const *V, const double *coef, int k,
                               cudaStream_t s);
 cudaError_t launch_scale_copy(int n, const double *src, double alpha, double *dst, cudaStream_t s);
+// dst = src / sqrt(*norm2), norm2 on the device
+cudaError_t launch_normalise(int n, const double *src, const double *norm2, double *dst,
+                             cudaStream_t s);
 cudaError_t launch_sub(int n, const double *a, const double *b, double *out, cudaStream_t s);
 
 }  // namespace rt3d
