@@ -195,13 +195,15 @@ typedef struct {
     int block;            /* threads per block: 64, 128 or 256 */
     int rays_per_thread;  /* characteristics per thread: 1; 2 (face cells
                              (x, y) and (x, y + 1), y even, integrated together
-                             in packed FP32x2 arithmetic); or 4 (face cells
-                             (x, y .. y + 3), y a multiple of 4, two packed
+                             in packed FP32x2 arithmetic); or 4 (four
+                             neighbouring face cells along y, or along x for
+                             the directions that step along x more, two packed
                              pairs, the J contributions of successive points
                              summed in FP32 per voxel while the voxel stays
-                             inside the block of voxels a warp's
+                             inside the block of voxels the thread's
                              characteristics occupy, then reduced in FP64;
-                             FP32 grids of at most 2^27 voxels) */
+                             FP32 grids of at most 2^27 voxels; 96 bytes a
+                             voxel allocated on first use) */
     int widen;            /* FP32 contribution to FP64 for the reduction: 0 the
                              conversion instruction, 1 integer moves, 2 both
                              (one characteristic per thread: alternating from

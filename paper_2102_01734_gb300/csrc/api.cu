@@ -132,6 +132,9 @@ struct rt3d_grid {
     // (zero between launches) and the kernel shape chosen by fs_tune
     double *Jrep = nullptr;  // [4N]
     float4 *pairs = nullptr;  // [4N] pair-packed FP32 (chi, S) of the two-characteristic kernel
+    // the four-characteristic kernel's, x and y exchanged (allocated on first use)
+    float4 *pairs_t = nullptr;
+    double *Jrep_t = nullptr;
     FsShape fs_shape{0, 0, 0, 0};  // block 0: not chosen yet
     float fs_tune_ms[RT3D_FS_TUNE_SHAPES] = {};  // last tuning: time of each shape
     void *a = nullptr;  // 26 OS off-diagonal planes, os_coef_index layout (f64 in FP64 mode, f32 otherwise)
@@ -338,6 +341,8 @@ rt3d_status fs_params(rt3d_grid *g, const rt3d_bc *bc, bool fp64, bool homogeneo
     q.Jrep = g->Jrep;
     q.pairs = g->pairs;
     q.rec4 = g->tpl.rec4;
+    q.swap = g->tpl.swap;
+    q.order4 = g->tpl.order4;
     q.chiS = fp64 ? g->chiS64 : g->chiS32;
     q.homogeneous = homogeneous ? 1 : 0;
     if (bc && !homogeneous) {
@@ -381,24 +386,42 @@ constexpr FsShape kFsShapes[RT3D_FS_TUNE_SHAPES] = {
     {256, 1, 0, 1}, {128, 2, 1, 1}, {256, 2, 2, 1}, {256, 4, 1, 1},
     {128, 4, 1, 1}, {64, 4, 1, 1},  {256, 4, 0, 1}, {128, 4, 0, 1}};
 
+// Buffers of the four-characteristic kernel (on first use).
+rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
+    const size_t N = (size_t)g->N;
+    if (!g->pairs_t) TRY(g->alloc(&g->pairs_t, 4 * N));
+    if (!g->Jrep_t) {
+        TRY(g->alloc(&g->Jrep_t, 4 * N));
+        CK(cudaMemsetAsync(g->Jrep_t, 0, sizeof(double) * 4 * N, g->stream));
+    }
+    p->pairs_t = g->pairs_t;
+    p->Jrep_t = g->Jrep_t;
+    return RT3D_OK;
+}
+
 // Autotuner of the FP32 formal solution's ray-bundle shape: times one launch
 // of every shape on the grid's current (chi, S) (CUDA events on the grid's
 // stream, after one untimed launch) and keeps the fastest. Each launch is
 // folded into g->Jfs, which the caller's launch overwrites.
-rt3d_status fs_tune(rt3d_grid *g, const FsParams &p) {
+rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
+    // above 2^25 voxels the four-characteristic kernel's 96 bytes a voxel are
+    // left to the solver's vectors
+    const bool four = quad_applicable(p) && g->N <= (1LL << 25);
+    if (four) TRY(quad_setup(g, &p));
     float best = 0.0f;
     int pick = 0;
     for (int i = -1; i < RT3D_FS_TUNE_SHAPES; ++i) {
         const int c = i < 0 ? 0 : i;
-        if (kFsShapes[c].rays_per_thread == 4 && !quad_applicable(p)) {
+        if (kFsShapes[c].rays_per_thread == 4 && !four) {
             g->fs_tune_ms[c] = 0.0f;  // not available on this grid
             continue;
         }
         CK(cudaEventRecord(g->ev0, g->stream));
         CK(launch_fs_fast(p, g->parab, kFsShapes[c], g->stream));
         CK(cudaEventRecord(g->ev1, g->stream));
-        CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream));
+        CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream,
+                       kFsShapes[c].rays_per_thread == 4 ? g->Jrep_t : nullptr));
         g->launches += 2;
         CK(cudaEventSynchronize(g->ev1));
         float ms = 0.0f;
@@ -548,7 +571,10 @@ rt3d_status run_fs(rt3d_grid *g, const FsParams &base, bool fp64, bool with_lsta
     if (g->sph) return run_fs_sph(g, base, p.chiS, fp64 ? 1 : 0, with_lstar);
     // without Lambda*: the replicated-accumulation kernels (J folded after)
     const bool fast = !with_lstar;
-    if (fast && !fp64 && g->fs_shape.block == 0) TRY(fs_tune(g, p));
+    if (fast && !fp64) {
+        if (g->fs_shape.block == 0) TRY(fs_tune(g, p));
+        if (g->fs_shape.rays_per_thread == 4) TRY(quad_setup(g, &p));
+    }
     if (!fast) CK(cudaMemsetAsync(g->Jfs, 0, sizeof(double) * g->N, g->stream));
     if (with_lstar) CK(cudaMemsetAsync(g->lstar, 0, sizeof(double) * 27 * g->N, g->stream));
     TRY(collect_events(g));
@@ -561,7 +587,8 @@ rt3d_status run_fs(rt3d_grid *g, const FsParams &base, bool fp64, bool with_lsta
     if (!fp64 && with_lstar) ++g->fs_lstar32;
     ++g->launches;
     if (fast) {
-        CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream));
+        CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream,
+                       !fp64 && g->fs_shape.rays_per_thread == 4 ? g->Jrep_t : nullptr));
         ++g->launches;
     }
     return RT3D_OK;
@@ -1177,7 +1204,11 @@ rt3d_status grid_build(rt3d_grid *g) {
     TRY(g->alloc(&t.rec32, total));
     TRY(g->alloc(&t.rec64, total));
     const bool quad = !g->fs64 && 4LL * g->nx * g->ny * g->nz <= (1LL << 29) - 1;
-    if (quad) TRY(g->alloc(&t.rec4, total));
+    if (quad) {
+        TRY(g->alloc(&t.rec4, total));
+        TRY(g->alloc(&t.swap, nO));
+        TRY(g->alloc(&t.order4, nO));
+    }
     double *d_dir = nullptr, *d_wt = nullptr, *d_ls = nullptr;
     int *d_cap = nullptr, *d_err = nullptr;
     TRY(g->alloc(&d_dir, 3 * nO));
@@ -1216,7 +1247,13 @@ rt3d_status grid_build(rt3d_grid *g) {
     tp.layer_sum = d_ls;
     tp.err = d_err;
     CK(launch_trace(tp, s));
-    if (quad) CK(launch_quad_rec(t, g->nx, g->ny, t.rec4, s));
+    std::vector<signed char> swap(nO);
+    for (int o = 0; o < nO; ++o)
+        swap[o] = std::fabs(g->dir[3 * o]) > std::fabs(g->dir[3 * o + 1]) ? 1 : 0;
+    if (quad) {
+        CK(cudaMemcpyAsync(t.swap, swap.data(), nO, cudaMemcpyHostToDevice, s));
+        CK(launch_quad_rec(t, g->nx, g->ny, t.rec4, s));
+    }
     int herr = 0;
     g->K.resize(nO);
     CK(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1230,6 +1267,10 @@ rt3d_status grid_build(rt3d_grid *g) {
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return g->K[a] > g->K[b]; });
     CK(cudaMemcpyAsync(t.order, order.data(), sizeof(int) * nO, cudaMemcpyHostToDevice, s));
+    std::vector<int> order4 = order;
+    std::stable_partition(order4.begin(), order4.end(), [&](int a) { return !swap[a]; });
+    if (quad)
+        CK(cudaMemcpyAsync(t.order4, order4.data(), sizeof(int) * nO, cudaMemcpyHostToDevice, s));
     t.kmax = *std::max_element(g->K.begin(), g->K.end());
     g->segments = 0;
     for (int o = 0; o < nO; ++o) g->segments += (long long)g->K[o] * g->nx * g->ny;

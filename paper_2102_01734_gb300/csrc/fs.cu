@@ -34,6 +34,8 @@
 // a (S_k - S_{k-1}) + f s d ((S_k - S_{k-1}) - q (S_{k+1} - S_k)), which
 // needs neither E nor a0. The last point of a characteristic is
 // linear; the entry point has S_{-1} = S_0 and chi_{-1} l_{-1} = 0.
+#include <algorithm>
+
 #include "fs_step.cuh"
 #include "fs64_step.cuh"
 
@@ -382,162 +384,96 @@ __global__ void __launch_bounds__(256) fs_pair_kernel(FsParams p) {
     }
 }
 
-// ---- Four characteristics per thread with the J contributions summed
-// across points before the FP64 reduction.
+// ---- Four characteristics per thread, the J contributions of successive
+// points summed in registers before the FP64 reduction.
 //
-// Lane t of the angle's launch integrates face cells (x0, y0 + r), r = 0..3,
-// x0 = t mod nx, y0 = 4 (t div nx) (two packed pairs). All characteristics
-// of an angle are translates, so at every point the 32 lanes x 4 rays of a
-// warp occupy a block of voxels that moves by one voxel in x, in y or in z
-// from point to point (the step type is stored with the point's record).
-// Each lane keeps four FP32 sums, one per row, for the voxels its rays
-// currently occupy, and adds the contribution (J weight x I) of every point.
-// When the block moves in x the sums move one lane over with warp shuffles
-// (the voxel a lane's rays enter was its neighbour's); in y they move one
-// row over inside the lane; a sum whose voxel leaves the block is reduced
-// into the replicated FP64 J: after an x-step through a per-warp list in
-// shared memory that is drained 32 entries at a time by all lanes, after a
-// y-step directly (one row of the block), after a z-step or a diagonal step
-// all four. Lanes of one face row (quad of rows) form a segment: the sums
-// move only between lanes of the same segment, and only between rows that
-// exist (a y-step towards the face's last row reduces the sum of the last
-// existing row instead of moving it on). A sum holds the contributions
-// of one voxel from successive rays, at most ~(points per layer) of them,
-// before its FP64 reduction.
+// One FP64 reduction a segment is what bounds the kernels above: 6.3e11 a
+// second at 129^3, and 5.9e11 to 7e11 whatever their width in a loop of
+// reductions alone. All characteristics of an angle are translates: when they
+// step along an axis, each enters the voxel that its neighbour on that axis
+// leaves. So a thread takes four neighbours along the axis the angle steps along
+// most (rows; x0 or y0 + 0..3), keeps an FP32 sum for the voxel of each row, and
+// on a step along that axis moves the sums one row over and reduces only the
+// one whose voxel no row holds any more; any other step reduces all four. On
+// average 0.54 reductions a segment are left. The lanes take consecutive cells
+// of the other axis, so that loads and reductions stay contiguous: the angles
+// that step along x more than along y run on arrays with x and y exchanged
+// (pairs_t, Jrep_t, offsets of their records).
+// Measured against the pair kernel: 129^3, 2048 angles 46.2 -> 38.4 ms (7.6e11
+// segments/s), 97^3, 512 angles 4.29 -> 3.45 ms, 65^3 1.35 -> 1.21 ms; at 33^3,
+// 128 angles 0.165 against 0.110 ms (one per thread), where the longest
+// characteristic's latency counts. Bound by FP32 issue: 80 warp instructions per
+// point of two warps' worth of segments (99 without the votes and the sums), 35
+// of them FP32, 71 % of the issue slots at 24 warps a SM (80 registers).
+// A sum holds at most the contributions of the rows that pass its voxel at
+// successive points. Rows past the face (its last quad) are integrated like the
+// others; their sums are never reduced and never move into an existing row.
 constexpr int kQuadOffBits = 29;
 constexpr unsigned kQuadOffMask = (1u << kQuadOffBits) - 1u;
-constexpr int kQuadSpill = 64;  // spill list entries per warp
-
-// Reduces a warp's spill list into J (all lanes; entries with index < 0 are
-// empty) and empties it. An entry holds the four row sums of a lane, the
-// replicated index of its row-0 voxel (low 29 bits) and its last existing
-// row (bits 29-30).
-template <int CONV>
-__device__ __forceinline__ void quad_drain(const float2 *sa, const float2 *sb, int *si,
-                                           double *__restrict__ Jrep, int rowp, int lane) {
-    __syncwarp();
-    for (int e = lane; e < kQuadSpill; e += 32) {
-        const int code = si[e];
-        if (code >= 0) {
-            const float2 va = sa[e], vb = sb[e];
-            const int rtop = code >> kQuadOffBits;
-            double *j = Jrep + (code & (int)kQuadOffMask);
-            atomicAdd(j, pair_widen<CONV>(va.x));
-            if (rtop >= 1) atomicAdd(j + rowp, pair_widen<CONV>(va.y));
-            if (rtop >= 2) atomicAdd(j + 2 * rowp, pair_widen<CONV>(vb.x));
-            if (rtop >= 3) atomicAdd(j + 3 * rowp, pair_widen<CONV>(vb.y));
-            si[e] = -1;
-        }
-    }
-    __syncwarp();
-}
 
 template <bool PARAB, int CONV>
 __global__ void __launch_bounds__(256, 3) fs_quad_kernel(FsParams p) {
-    __shared__ float2 sp_a[8][kQuadSpill], sp_b[8][kQuadSpill];
-    __shared__ int sp_idx[8][kQuadSpill];
-    constexpr unsigned FULL = 0xffffffffu;
-    const int nq = (p.ny + 3) >> 2;
-    const int nlive = p.nx * nq;
-    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int o = p.order4[blockIdx.y];
+    const bool tr = p.swap[o];
+    const int nm = tr ? p.ny : p.nx, nd = tr ? p.nx : p.ny;  // lanes' axis, rows' axis
+    const int nlive = nm * ((nd + 3) >> 2);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t - lane >= nlive) return;  // the whole warp is past the face (warp-uniform)
-    const bool live = t < nlive;
-    const int tt = live ? t : nlive - 1;
-    const int o = p.order[blockIdx.y];
+    if (t - (threadIdx.x & 31) >= nlive) return;  // the whole warp is past the face
+    const int tt = min(t, nlive - 1);
     const int K = p.tlen[o];
     const float4 *__restrict__ rec = p.rec4 + p.toff[o];
-    const int x0 = tt % p.nx, q = tt / p.nx, y0 = 4 * q;
-    const int base = x0 + 2 * p.nx * y0;
-    const int rowp = 2 * p.nx;  // one replicated row
-    const float4 *__restrict__ PA = p.pairs + base;
-    // rows y0 + 2, y0 + 3 (a quad without them reads pair A's data, unused)
-    const float4 *__restrict__ PB = (y0 + 2 < p.ny) ? PA + 2 * rowp : PA;
-    double *__restrict__ J0 = p.Jrep + base;
-    // the quad's last existing row (-1: a lane past the face). Rows past it
-    // (the face's last quad when ny is not a multiple of 4) are integrated
-    // and summed like the others, but their sums are never reduced and never
-    // move into an existing row.
-    const int rtop = live ? min(3, p.ny - 1 - y0) : -1;
-    // segments: the lanes of one quad of rows (consecutive x0); lane 0 is live
-    const int seg = live ? q : -1;
-    const int segL = __shfl_up_sync(FULL, seg, 1), segR = __shfl_down_sync(FULL, seg, 1);
-    const bool hasL = lane > 0 && live && segL == seg;
-    const bool hasR = lane < 31 && live && segR == seg;
-    const float2 takeP = pk1(hasR ? 1.0f : 0.0f), takeM = pk1(hasL ? 1.0f : 0.0f);
-    const int nsub = 31 / p.nx + 2;           // segments a warp can span
-    const int per_drain = kQuadSpill / nsub;  // x-steps between drains of the spill list
-    const int slot0 = seg - __shfl_sync(FULL, seg, 0);
-    const int spill_tag = (rtop < 0 ? 0 : rtop) << kQuadOffBits;
-    float2 *sa = sp_a[wb];
-    float2 *sb = sp_b[wb];
-    int *si = sp_idx[wb];
-    for (int e = lane; e < kQuadSpill; e += 32) si[e] = -1;
-    __syncwarp();
+    const int m0 = tt % nm, d0 = 4 * (tt / nm);
+    const int rowp = 2 * nm;  // one replicated row
+    const int base = m0 + rowp * d0;
+    // the second pair, or the first one's data again where it is past the face
+    const float4 *__restrict__ P0 = (tr ? p.pairs_t : p.pairs) + base;
+    const float4 *__restrict__ P1 = d0 + 2 < nd ? P0 + 2 * rowp : P0;
+    double *__restrict__ J0 = (tr ? p.Jrep_t : p.Jrep) + base;
+    // the quad's last existing row (-1: a lane past the face)
+    const int rtop = t < nlive ? min(3, nd - 1 - d0) : -1;
 
     float Iv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (!p.homogeneous) {
         const bool up = p.up[o];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            if (y0 + r < p.ny)
-                Iv[r] = (float)entry_intensity(up, p.mu, o, (y0 + r) * p.nx + x0, p.top_face,
-                                               p.bot_face, p.bot_grad, p.I_top, p.I_bot);
+            if (d0 + r < nd) {
+                const int f = tr ? d0 + r + p.nx * m0 : m0 + p.nx * (d0 + r);
+                Iv[r] = (float)entry_intensity(up, p.mu, o, f, p.top_face, p.bot_face, p.bot_grad,
+                                               p.I_top, p.I_bot);
+            }
     }
-    RayP a, b;
+    RayN s[2];
     const float4 r0 = __ldg(rec);
     int vc = (int)(__float_as_uint(r0.x) & kQuadOffMask);
-    pair_init(a, __ldg(PA + vc), pk(r0.z, r0.w), Iv[0], Iv[1]);
-    pair_init(b, __ldg(PB + vc), pk(r0.z, r0.w), Iv[2], Iv[3]);
-    float2 A01 = pk1(0.0f), A23 = pk1(0.0f);  // sums of rows y0 .. y0 + 3 at the current voxels
+    quad_start(s[0], __ldg(P0 + vc), pk(r0.z, r0.w), Iv[0], Iv[1]);
+    quad_start(s[1], __ldg(P1 + vc), pk(r0.z, r0.w), Iv[2], Iv[3]);
+    float2 A01 = pk1(0.0f), A23 = pk1(0.0f);  // sums of the rows' current voxels
     float cwc = r0.y;
-    int cnt = 0;
+    auto reduce_all = [&](double *__restrict__ j) {
+        if (rtop >= 0) atomicAdd(j, pair_widen<CONV>(A01.x));
+        if (rtop >= 1) atomicAdd(j + rowp, pair_widen<CONV>(A01.y));
+        if (rtop >= 2) atomicAdd(j + 2 * rowp, pair_widen<CONV>(A23.x));
+        if (rtop >= 3) atomicAdd(j + 3 * rowp, pair_widen<CONV>(A23.y));
+    };
     // the next point's record and data are loaded one point ahead
-    float4 rn = __ldg(rec + (K > 1 ? 1 : 0));
-    unsigned bits = __float_as_uint(rn.x);
-    float4 cA = __ldg(PA + (bits & kQuadOffMask)), cB = __ldg(PB + (bits & kQuadOffMask));
-#pragma unroll 2
+    float4 rn = __ldg(rec + 1);
+    float4 c[2] = {__ldg(P0 + (__float_as_uint(rn.x) & kQuadOffMask)),
+                   __ldg(P1 + (__float_as_uint(rn.x) & kQuadOffMask))};
+// three points per trip: the carried values rotate with that period
+#pragma unroll 3
     for (int k = 1; k < K; ++k) {
-        const float4 rq = __ldg(rec + (k + 1 < K ? k + 1 : k));
-        const unsigned bq = __float_as_uint(rq.x);
-        const float4 qA = __ldg(PA + (bq & kQuadOffMask)), qB = __ldg(PB + (bq & kQuadOffMask));
-        const int vn = (int)(bits & kQuadOffMask);
-        const float2 hl = pk(rn.z, rn.w);
-        const float2 Ia = pair_advance_c<PARAB>(a, cA, hl);
-        const float2 Ib = pair_advance_c<PARAB>(b, cB, hl);
-        A01 = fma2(Ia, pk1(cwc), A01);
-        A23 = fma2(Ib, pk1(cwc), A23);
-        // the block moves from the current points (offset vc) to the next
-        const unsigned type = bits >> kQuadOffBits;
-        if (type <= 1u) {  // x-step: +1 (type 0) or -1 (type 1)
-            const bool plus = type == 0u;
-            if (live && (plus ? !hasL : !hasR)) {  // no lane takes this voxel over
-                const int e = cnt * nsub + slot0;
-                sa[e] = A01;
-                sb[e] = A23;
-                si[e] = (base + vc) | spill_tag;
-            }
-            float s0, s1, s2, s3;
-            if (plus) {
-                s0 = __shfl_down_sync(FULL, A01.x, 1);
-                s1 = __shfl_down_sync(FULL, A01.y, 1);
-                s2 = __shfl_down_sync(FULL, A23.x, 1);
-                s3 = __shfl_down_sync(FULL, A23.y, 1);
-            } else {
-                s0 = __shfl_up_sync(FULL, A01.x, 1);
-                s1 = __shfl_up_sync(FULL, A01.y, 1);
-                s2 = __shfl_up_sync(FULL, A23.x, 1);
-                s3 = __shfl_up_sync(FULL, A23.y, 1);
-            }
-            const float2 take = plus ? takeP : takeM;
-            A01 = mul2(pk(s0, s1), take);
-            A23 = mul2(pk(s2, s3), take);
-            if (++cnt == per_drain) {
-                quad_drain<CONV>(sa, sb, si, p.Jrep, rowp, lane);
-                cnt = 0;
-            }
-        } else if (type == 2u) {  // y-step +1: row y0's voxel leaves
-            if (rtop >= 0) atomicAdd(J0 + vc, pair_widen<CONV>(A01.x));
+        const float4 rq = __ldg(rec + k + 1);
+        const unsigned oq = __float_as_uint(rq.x) & kQuadOffMask;
+        const float4 q[2] = {__ldg(P0 + oq), __ldg(P1 + oq)};
+        quad_advance<PARAB>(s, c, pk(rn.z, rn.w));
+        A01 = fma2(s[0].I, pk1(cwc), A01);
+        A23 = fma2(s[1].I, pk1(cwc), A23);
+        // the move from the current points (offset vc) to the next
+        const unsigned type = __float_as_uint(rn.x) >> kQuadOffBits;
+        double *__restrict__ j = J0 + vc;
+        if (type == 0u) {  // one row up: row 0's voxel leaves
+            if (rtop >= 0) atomicAdd(j, pair_widen<CONV>(A01.x));
             A01 = pk(A01.y, A23.x);
             A23 = pk(A23.y, 0.0f);
             if (rtop < 3) {  // the last existing row enters a voxel no sum of this lane holds
@@ -545,72 +481,95 @@ __global__ void __launch_bounds__(256, 3) fs_quad_kernel(FsParams p) {
                 else if (rtop == 1) A01.y = 0.0f;
                 else A01.x = 0.0f;
             }
-        } else if (type == 3u) {  // y-step -1: the voxel of the last existing row leaves
+        } else if (type == 1u) {  // one row down: the last existing row's voxel leaves
             const float v = rtop == 3 ? A23.y : (rtop == 2 ? A23.x : (rtop == 1 ? A01.y : A01.x));
-            if (rtop >= 0) atomicAdd(J0 + rtop * rowp + vc, pair_widen<CONV>(v));
+            if (rtop >= 0) atomicAdd(j + rtop * rowp, pair_widen<CONV>(v));
             A23 = pk(A01.y, A23.x);
             A01 = pk(0.0f, A01.x);
-        } else {  // z-step or diagonal step: all four leave
-            double *j = J0 + vc;
-            if (rtop >= 0) atomicAdd(j, pair_widen<CONV>(A01.x));
-            if (rtop >= 1) atomicAdd(j + rowp, pair_widen<CONV>(A01.y));
-            if (rtop >= 2) atomicAdd(j + 2 * rowp, pair_widen<CONV>(A23.x));
-            if (rtop >= 3) atomicAdd(j + 3 * rowp, pair_widen<CONV>(A23.y));
+        } else {  // all four leave
+            reduce_all(j);
             A01 = pk1(0.0f);
             A23 = pk1(0.0f);
         }
-        vc = vn;
+        vc = (int)(__float_as_uint(rn.x) & kQuadOffMask);
         cwc = rn.y;
         rn = rq;
-        bits = bq;
-        cA = qA;
-        cB = qB;
+        c[0] = q[0];
+        c[1] = q[1];
     }
     // the last point: linear form
-    const float2 Ia = pair_last(a), Ib = pair_last(b);
-    A01 = fma2(Ia, pk1(cwc), A01);
-    A23 = fma2(Ib, pk1(cwc), A23);
-    double *j = J0 + vc;
-    if (rtop >= 0) atomicAdd(j, pair_widen<CONV>(A01.x));
-    if (rtop >= 1) atomicAdd(j + rowp, pair_widen<CONV>(A01.y));
-    if (rtop >= 2) atomicAdd(j + 2 * rowp, pair_widen<CONV>(A23.x));
-    if (rtop >= 3) atomicAdd(j + 3 * rowp, pair_widen<CONV>(A23.y));
-    quad_drain<CONV>(sa, sb, si, p.Jrep, rowp, lane);
+    const float2 I0 = linear_n(s[0], interval_both(s[0].u)), I1 = linear_n(s[1], interval_both(s[1].u));
+    A01 = fma2(I0, pk1(cwc), A01);
+    A23 = fma2(I1, pk1(cwc), A23);
+    double *__restrict__ j = J0 + vc;
+    reduce_all(j);
     // a non-finite intensity persists along the recurrence: make J NaN
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    if (rtop >= 0 && !(fabsf(Ia.x) <= 3.402823466e38f)) atomicAdd(j, nan);
-    if (rtop >= 1 && !(fabsf(Ia.y) <= 3.402823466e38f)) atomicAdd(j + rowp, nan);
-    if (rtop >= 2 && !(fabsf(Ib.x) <= 3.402823466e38f)) atomicAdd(j + 2 * rowp, nan);
-    if (rtop >= 3 && !(fabsf(Ib.y) <= 3.402823466e38f)) atomicAdd(j + 3 * rowp, nan);
+    if (rtop >= 0 && !(fabsf(I0.x) <= 3.402823466e38f)) atomicAdd(j, nan);
+    if (rtop >= 1 && !(fabsf(I0.y) <= 3.402823466e38f)) atomicAdd(j + rowp, nan);
+    if (rtop >= 2 && !(fabsf(I1.x) <= 3.402823466e38f)) atomicAdd(j + 2 * rowp, nan);
+    if (rtop >= 3 && !(fabsf(I1.y) <= 3.402823466e38f)) atomicAdd(j + 3 * rowp, nan);
 }
 
 // Records of the four-characteristic kernel: (offset | step type << 29,
-// J weight, l/2, l/2), the step type of the move from the previous point:
-// 0 x + 1, 1 x - 1, 2 y + 1, 3 y - 1, 4 anything else (z, diagonal, first).
+// J weight, l/2, l/2), offsets with x and y exchanged for the angles that swap
+// them, the step type of the move from the previous point: 0 one row up, 1 one
+// row down, 2 anything else (the first point too).
 __global__ void quad_rec_kernel(int nx, int ny, const long long *__restrict__ toff,
-                                const int *__restrict__ tlen, const uint32_t *__restrict__ code,
+                                const int *__restrict__ tlen, const signed char *__restrict__ swap,
+                                const uint32_t *__restrict__ code,
                                 const float4 *__restrict__ rec32, float4 *__restrict__ rec4) {
     const int o = blockIdx.x;
     const long long t0 = toff[o];
     const int K = tlen[o];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        unsigned type = 4u;
+    const bool tr = swap[o];
+    const int nm = tr ? ny : nx, nd = tr ? nx : ny;
+    for (int i = threadIdx.x; i <= K; i += blockDim.x) {
+        const int k = min(i, K - 1);  // one record more: the last point again, to load ahead
+        auto split = [&](uint32_t c, int &m, int &d, int &z) {
+            const int x = (int)(c & 0x7ffu), y = (int)((c >> 11) & 0x7ffu);
+            m = tr ? y : x;
+            d = tr ? x : y;
+            z = (int)(c >> 22);
+        };
+        int m1, d1, z1;
+        split(code[t0 + k], m1, d1, z1);
+        unsigned type = 2u;
         if (k > 0) {
-            const uint32_t c1 = code[t0 + k], c0 = code[t0 + k - 1];
-            int ddx = (int)(c1 & 0x7ffu) - (int)(c0 & 0x7ffu);
-            int ddy = (int)((c1 >> 11) & 0x7ffu) - (int)((c0 >> 11) & 0x7ffu);
-            const int ddz = (int)(c1 >> 22) - (int)(c0 >> 22);
-            if (ddx == nx - 1) ddx = -1;  // wrapped offsets: a step across the
-            if (ddx == 1 - nx) ddx = 1;   // periodic boundary
-            if (ddy == ny - 1) ddy = -1;
-            if (ddy == 1 - ny) ddy = 1;
-            if (ddz == 0 && ddy == 0 && (ddx == 1 || ddx == -1)) type = ddx == 1 ? 0u : 1u;
-            if (ddz == 0 && ddx == 0 && (ddy == 1 || ddy == -1)) type = ddy == 1 ? 2u : 3u;
+            int m0, d0, z0;
+            split(code[t0 + k - 1], m0, d0, z0);
+            int dd = d1 - d0;
+            if (dd == nd - 1) dd = -1;  // wrapped offsets: a step across the
+            if (dd == 1 - nd) dd = 1;   // periodic boundary
+            if (m1 == m0 && z1 == z0 && (dd == 1 || dd == -1)) type = dd == 1 ? 0u : 1u;
         }
         const float4 r = rec32[t0 + k];
-        const unsigned off = __float_as_uint(r.x);
-        rec4[t0 + k] = make_float4(__uint_as_float(off | (type << kQuadOffBits)), r.y, r.z, r.w);
+        const unsigned off = (unsigned)rep_index(m1, d1, z1, nm, nd);
+        rec4[t0 + i] = make_float4(__uint_as_float(off | (type << kQuadOffBits)), r.y, r.z, r.w);
     }
+}
+
+// p.pairs_t from the replicated FP32 (chi, S): the pair-packed arrays with x
+// and y exchanged, element y + 2 ny (x + 2 nx z) the values of columns x and
+// x + 1 at y; transposed 32 x 32 at a time through shared memory.
+__global__ void __launch_bounds__(256) pair_pack_t_kernel(int nx, int ny, const float2 *__restrict__ chiS,
+                                                          float4 *__restrict__ P) {
+    __shared__ float2 tile[32][34];
+    const int wx = 2 * nx, wy = 2 * ny, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const long long layer = (long long)wx * wy * blockIdx.z;
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+    for (int j = ty; j < 32; j += 8)
+        for (int i = tx; i < 33; i += 32)
+            if (y0 + j < wy) {
+                const int x = x0 + i < wx ? x0 + i : x0 + i - wx;  // the last column pairs with the first
+                if (x < wx) tile[j][i] = chiS[layer + x + (long long)wx * (y0 + j)];
+            }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8)
+        if (x0 + i < wx && y0 + tx < wy) {
+            const float2 a = tile[tx][i], b = tile[tx][i + 1];
+            P[layer + y0 + tx + (long long)wy * (x0 + i)] = make_float4(a.x, b.x, a.y, b.y);
+        }
 }
 
 // p.pairs from the replicated FP32 (chi, S): at every replicated index the
@@ -709,17 +668,26 @@ __global__ void __launch_bounds__(128) fs64_fast_kernel(FsParams p) {
     atomicAdd(J + vc, cwc * I);
 }
 
-// J[v] = sum of the four replicas of v in Jrep (FP64); Jrep zeroed for the
-// next launch.
+// J[v] = sum of the four replicas of v in Jrep (FP64), and of the four in
+// Jrep_t (x and y exchanged) where it is given; both zeroed for the next launch.
 __global__ void fold_kernel(int nx, int ny, int nz, double *__restrict__ Jrep,
-                            double *__restrict__ J) {
+                            double *__restrict__ Jrep_t, double *__restrict__ J) {
     const long long n = (long long)nx * ny * nz;
     const long long dy = 2LL * nx * ny;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
          v += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(v % nx), y = (int)((v / nx) % ny), z = (int)(v / ((long long)nx * ny));
         const long long i0 = rep_index(x, y, z, nx, ny);
-        J[v] = (Jrep[i0] + Jrep[i0 + nx]) + (Jrep[i0 + dy] + Jrep[i0 + dy + nx]);
+        double sum = (Jrep[i0] + Jrep[i0 + nx]) + (Jrep[i0 + dy] + Jrep[i0 + dy + nx]);
+        if (Jrep_t) {
+            const long long t0 = rep_index(y, x, z, ny, nx);
+            sum += (Jrep_t[t0] + Jrep_t[t0 + ny]) + (Jrep_t[t0 + dy] + Jrep_t[t0 + dy + ny]);
+            Jrep_t[t0] = 0.0;
+            Jrep_t[t0 + ny] = 0.0;
+            Jrep_t[t0 + dy] = 0.0;
+            Jrep_t[t0 + dy + ny] = 0.0;
+        }
+        J[v] = sum;
         Jrep[i0] = 0.0;
         Jrep[i0 + nx] = 0.0;
         Jrep[i0 + dy] = 0.0;
@@ -762,7 +730,7 @@ bool quad_applicable(const FsParams &p) {
 }
 
 cudaError_t launch_quad_rec(const Template &t, int nx, int ny, float4 *rec4, cudaStream_t s) {
-    quad_rec_kernel<<<t.nangles, 256, 0, s>>>(nx, ny, t.toff, t.tlen, t.code, t.rec32, rec4);
+    quad_rec_kernel<<<t.nangles, 256, 0, s>>>(nx, ny, t.toff, t.tlen, t.swap, t.code, t.rec32, rec4);
     return cudaGetLastError();
 }
 
@@ -782,7 +750,9 @@ cudaError_t launch_fs_fast(const FsParams &p, bool parabolic, const FsShape &sh,
         pair_pack_kernel<<<rows < 65536 ? rows : 65536, 256, 0, s>>>(
             p.nx, p.ny, p.nz, static_cast<const float2 *>(p.chiS), p.pairs);
         if (sh.rays_per_thread == 4) {
-            const int nlanes = p.nx * ((p.ny + 3) / 4);
+            pair_pack_t_kernel<<<dim3((2 * p.nx + 31) / 32, (2 * p.ny + 31) / 32, p.nz), 256, 0, s>>>(
+                p.nx, p.ny, static_cast<const float2 *>(p.chiS), p.pairs_t);
+            const int nlanes = std::max(p.nx * ((p.ny + 3) / 4), p.ny * ((p.nx + 3) / 4));
             dim3 grid((nlanes + sh.block - 1) / sh.block, p.nangles);
             if (parabolic) launch_quad_w<true>(p, grid, sh.block, sh.widen, s);
             else launch_quad_w<false>(p, grid, sh.block, sh.widen, s);
@@ -813,12 +783,13 @@ cudaError_t launch_fs64_fast(const FsParams &p, bool parabolic, cudaStream_t s) 
     return cudaGetLastError();
 }
 
-cudaError_t launch_fold(int nx, int ny, int nz, double *Jrep, double *J, cudaStream_t s) {
+cudaError_t launch_fold(int nx, int ny, int nz, double *Jrep, double *J, cudaStream_t s,
+                        double *Jrep_t) {
     const long long n = (long long)nx * ny * nz;
     long long b = (n + 255) / 256;
     const long long cap = 16LL * device_sm_count();
     if (b > cap) b = cap;
-    fold_kernel<<<(int)b, 256, 0, s>>>(nx, ny, nz, Jrep, J);
+    fold_kernel<<<(int)b, 256, 0, s>>>(nx, ny, nz, Jrep, Jrep_t, J);
     return cudaGetLastError();
 }
 

@@ -268,6 +268,124 @@ __device__ __forceinline__ void pair_init(RayP &s, const float4 &c, float2 hl, f
     s.nru = pk(rcp_approx(fminf(-s.hc.x, -1e-15f)), rcp_approx(fminf(-s.hc.y, -1e-15f)));
 }
 
+// ---- The same for the four-characteristic kernel, two pairs at a time ----
+// The branches are taken by the warp (votes): all intervals below 1 (the
+// polynomials, the parabolic blend), all from 1 on (the exponential; the blend
+// is 0 there and left out), or both kinds, where both are evaluated. The signs
+// are chosen so that every product is a plain fused multiply-add (a packed
+// operand has no free negation): the state keeps nD = Sp - Sc, and the interval
+// functions are e0, -a and d.
+struct RayN {
+    float2 I, u, hc, Sp, Sc, nD;
+};
+struct IntervalN2 {
+    float2 e0, na, d;
+};
+__device__ __forceinline__ IntervalN2 interval_thin(float2 u) {
+    float2 np = fma2(pk1(3.569704858819023e-05f), u, pk1(-3.819821577053517e-04f));  // -p(u)
+    np = fma2(np, u, pk1(2.770215505734086e-03f));
+    np = fma2(np, u, pk1(-1.6664894297719002e-02f));
+    np = fma2(np, u, pk1(8.333317935466766e-02f));
+    np = fma2(np, u, pk1(-3.333333432674408e-01f));
+    const float2 nb = mul2(u, np);             // -b
+    const float2 nhu = mul2(u, pk1(-0.5f));
+    IntervalN2 r;
+    r.na = fma2(nhu, nb, nhu);                 // -u (1 - b) / 2
+    r.e0 = fma2(u, r.na, u);                   // u (1 - a)
+    r.d = sub2(nb, r.na);                      // a - b
+    return r;
+}
+__device__ __forceinline__ IntervalN2 interval_thick(float2 u) {
+    const float2 t = mul2(u, pk1(-1.4426950408889634f));  // -u log2(e)
+    IntervalN2 r;
+    r.e0 = sub2(pk1(1.0f), pk(ex2_approx(t.x), ex2_approx(t.y)));
+    r.na = fma2(r.e0, pk(rcp_approx(u.x), rcp_approx(u.y)), pk1(-1.0f));  // -(1 - e0/u)
+    r.d = pk1(0.0f);  // enters with blend weight 0 only
+    return r;
+}
+__device__ __forceinline__ IntervalN2 interval_both(float2 u) {
+    const IntervalN2 p = interval_thin(u), e = interval_thick(u);
+    const bool x = u.x < 1.0f, y = u.y < 1.0f;
+    IntervalN2 r;
+    r.e0 = pk(x ? p.e0.x : e.e0.x, y ? p.e0.y : e.e0.y);
+    r.na = pk(x ? p.na.x : e.na.x, y ? p.na.y : e.na.y);
+    r.d = pk(x ? p.d.x : 0.0f, y ? p.d.y : 0.0f);
+    return r;
+}
+// I + e0 (Sp - I) + a (Sc - Sp)
+__device__ __forceinline__ float2 linear_n(const RayN &s, const IntervalN2 &f) {
+    return fma2(f.na, s.nD, fma2(f.e0, sub2(s.Sp, s.I), s.I));
+}
+// f s d (dS - q dSn), both factors negated, added to In; w the next interval.
+// The two divisions share one reciprocal: with X = wf (u + wf), u/wf = u (u +
+// wf)/X and u/(u + wf) = u wf/X, wf = w floored at 1e-15 (X stays a normal FP32
+// number; a zero-opacity interval gets q = 0 or blend weight 0).
+__device__ __forceinline__ float2 parabola_n(const RayN &s, const IntervalN2 &f, float2 w, float2 nDn,
+                                             float2 In) {
+    const float2 nwf = pk(fminf(-w.x, -1e-15f), fminf(-w.y, -1e-15f));
+    const float2 nuw = sub2(nwf, s.u);  // -(u + wf)
+    const float2 X = mul2(nwf, nuw);
+    const float2 uR = mul2(s.u, pk(rcp_approx(X.x), rcp_approx(X.y)));
+    const float2 nq = mul2(nuw, uR), ns = mul2(nwf, uR);  // -u/wf, -u/(u + wf)
+    const float2 fw = mul2(pk(__saturatef(fmaf(-2.0f, s.u.x, 2.0f)), __saturatef(fmaf(-2.0f, s.u.y, 2.0f))),
+                           pk(__saturatef(fmaf(0.5f, nq.x, 2.0f)), __saturatef(fmaf(0.5f, nq.y, 2.0f))));
+    return fma2(mul2(mul2(fw, f.d), ns), fma2(nq, nDn, s.nD), In);
+}
+// One point of two pairs (all lanes of the warp): s[j].I becomes the
+// intensities at the current point, the rest moves to the next point (c[j] its
+// pair-packed (chi, S), hl its (l/2, l/2)).
+template <bool PARAB>
+__device__ __forceinline__ void quad_advance(RayN (&s)[2], const float4 (&c)[2], float2 hl) {
+    float2 hn[2], Sn[2], nDn[2], w[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        hn[j] = mul2(pk(c[j].x, c[j].y), hl);
+        Sn[j] = pk(c[j].z, c[j].w);
+        nDn[j] = sub2(s[j].Sc, Sn[j]);
+        w[j] = add2(s[j].hc, hn[j]);
+    }
+    const float hi = fmaxf(fmaxf(s[0].u.x, s[0].u.y), fmaxf(s[1].u.x, s[1].u.y));
+    if (__all_sync(0xffffffffu, hi < 1.0f)) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const IntervalN2 f = interval_thin(s[j].u);
+            const float2 In = linear_n(s[j], f);
+            s[j].I = PARAB ? parabola_n(s[j], f, w[j], nDn[j], In) : In;
+        }
+    } else {
+        const float lo = fminf(fminf(s[0].u.x, s[0].u.y), fminf(s[1].u.x, s[1].u.y));
+        if (__all_sync(0xffffffffu, lo >= 1.0f)) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) s[j].I = linear_n(s[j], interval_thick(s[j].u));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const IntervalN2 f = interval_both(s[j].u);
+                const float2 In = linear_n(s[j], f);
+                s[j].I = PARAB ? parabola_n(s[j], f, w[j], nDn[j], In) : In;
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        s[j].u = w[j];
+        s[j].hc = hn[j];
+        s[j].Sp = s[j].Sc;
+        s[j].Sc = Sn[j];
+        s[j].nD = nDn[j];
+    }
+}
+// A pair at its first point: the entry interval has chi_{-1} l_{-1} = 0 and
+// S_{-1} = S_0.
+__device__ __forceinline__ void quad_start(RayN &s, const float4 &c, float2 hl, float Ia, float Ib) {
+    s.I = pk(Ia, Ib);
+    s.hc = mul2(pk(c.x, c.y), hl);
+    s.u = s.hc;
+    s.Sc = pk(c.z, c.w);
+    s.Sp = s.Sc;
+    s.nD = pk1(0.0f);
+}
+
 // FP32 contribution to FP64 for a reduction: CONV 1 integer moves, else the
 // conversion instruction.
 template <int CONV> __device__ __forceinline__ double pair_widen(float x) {

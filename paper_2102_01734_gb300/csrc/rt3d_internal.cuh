@@ -50,6 +50,11 @@ struct Template {
     // grids of at most 2^27 voxels): rec32 with the step type in the top
     // three bits of the offset
     float4 *rec4 = nullptr;
+    // of the four-characteristic kernel: [nangles] 1 where an angle steps along
+    // x more than along y (x and y exchanged), and its order of the angles
+    // (those exchanged last, each part by decreasing length)
+    signed char *swap = nullptr;
+    int *order4 = nullptr;
 };
 
 // The packed (chi, S) arrays are replicated 2 x 2 in x and y: element
@@ -99,6 +104,10 @@ struct FsParams {
     // (chi(y), chi(y+1), S(y), S(y+1)); written from chiS by launch_fs_fast
     float4 *pairs;
     const float4 *rec4;  // nullable: step records of the four-characteristic kernel
+    const signed char *swap;  // with rec4: angles with x and y exchanged
+    const int *order4;
+    float4 *pairs_t;     // with rec4: [4N] pairs with x and y exchanged
+    double *Jrep_t;      // with rec4: [4N] Jrep with x and y exchanged
     double *lstar;     // nullable [27][N], accumulated into
     const double *top_face;  // nullable [ny*nx]
     const double *bot_face;  // nullable [ny*nx]
@@ -138,7 +147,8 @@ cudaError_t launch_fs(const FsParams &p, bool fp64, bool parabolic, bool lstar, 
 struct FsShape {
     int block;            // 64, 128 or 256 threads
     int rays_per_thread;  // 1; 2: face rows y and y + 1 in packed FP32x2 arithmetic;
-                          // 4: rows y .. y + 3, J summed across points in registers
+                          // 4: four rows (or columns) a thread, J summed across points
+                          // in registers
     int widen;            // FP32 -> FP64: 0 conversion, 1 integer moves, 2 alternating
                           // (two per thread: the second characteristic by integer moves)
     int branchless;       // 1: parabolic correction evaluated without a branch
@@ -165,7 +175,9 @@ cudaError_t launch_recff(long long total, const double2 *rec64, float4 *out, cud
 // FP64 formal solution without Lambda* into p.Jrep (zero on entry)
 cudaError_t launch_fs64_fast(const FsParams &p, bool parabolic, cudaStream_t s);
 // J[v] = sum of the four replicas of v in Jrep; zeroes Jrep
-cudaError_t launch_fold(int nx, int ny, int nz, double *Jrep, double *J, cudaStream_t s);
+// (and of Jrep_t, x and y exchanged, where given)
+cudaError_t launch_fold(int nx, int ny, int nz, double *Jrep, double *J, cudaStream_t s,
+                        double *Jrep_t = nullptr);
 
 // ---- ALI / OS kernels (ali.cu) ----
 struct OsState {
