@@ -209,10 +209,8 @@ typedef struct {
                              (one characteristic per thread: alternating from
                              point to point; two: the second by integer
                              moves; four: as 0) */
-    int branchless;       /* 1: the parabolic correction is evaluated without
-                             a branch (multiplied by its blend weight 0 where
-                             the linear form applies); two characteristics
-                             per thread always evaluate it so */
+    int branchless;       /* 0 or 1; no effect: the parabolic correction's
+                             branches are the kernel's own choice */
 } rt3d_fs_shape;
 
 #define RT3D_FS_TUNE_SHAPES 8

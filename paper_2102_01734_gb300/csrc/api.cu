@@ -376,15 +376,13 @@ rt3d_status collect_events(rt3d_grid *g) {
 }
 
 // Candidate shapes of the FP32 formal-solution kernel without Lambda* that
-// fs_tune times: (threads per block, characteristics per thread, widening,
-// branchless parabolic correction). Two characteristics per thread is the
-// packed FP32x2 kernel, four the packed kernel that sums J contributions in
-// registers before the FP64 reduction (both always branchless; widening 2 of
-// the four-characteristic kernel is the conversion, as 0). A grid where a
+// fs_tune times: (threads per block, characteristics per thread, widening, 1).
+// One characteristic per thread wins on small grids (33^3), where the longest
+// characteristic's latency counts, four on larger ones. A grid where a
 // candidate cannot run records 0 for it.
 constexpr FsShape kFsShapes[RT3D_FS_TUNE_SHAPES] = {
-    {256, 1, 0, 1}, {128, 2, 1, 1}, {256, 2, 2, 1}, {256, 4, 1, 1},
-    {128, 4, 1, 1}, {64, 4, 1, 1},  {256, 4, 0, 1}, {128, 4, 0, 1}};
+    {256, 1, 0, 1}, {128, 1, 1, 1}, {64, 1, 1, 1},  {128, 2, 1, 1},
+    {256, 4, 1, 1}, {128, 4, 1, 1}, {64, 4, 1, 1},  {64, 1, 2, 1}};
 
 // Buffers of the four-characteristic kernel (on first use).
 rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {

@@ -67,12 +67,11 @@ __global__ void b_source(int nx, int ny, int nz, const double *J, const double *
 }
 
 // FP32 formal solution (no Lambda*) of wavelength blockIdx.z into its
-// replicated FP64 J: the per-point step of the unbatched kernel (fast_step),
-// two points per trip, in the ray-bundle shape the batched autotuner chose
-// (threads per block from the launch; CONV as in fs_fast_kernel: 0 the
-// conversion instruction, 1 integer moves, 2 alternating; BL: parabolic
-// correction without a branch).
-template <bool PARAB, int CONV, bool BL>
+// replicated FP64 J: the unbatched kernel's characteristic (twin_ray), in the
+// ray-bundle shape the batched autotuner chose (threads per block from the
+// launch; CONV as in fs_fast_kernel: 0 the conversion instruction, 1 integer
+// moves, 2 alternating).
+template <bool PARAB, int CONV>
 __global__ void __launch_bounds__(256) b_fs(BatchFsParams p) {
     constexpr bool W0 = CONV == 1, W1 = CONV >= 1;
     if ((int)blockIdx.z >= p.bs->nactive) return;
@@ -90,37 +89,8 @@ __global__ void __launch_bounds__(256) b_fs(BatchFsParams p) {
     const double I0 = entry_intensity(p.up[o], p.mu, o, ray, p.top_face ? p.top_face + lf : nullptr,
                                       p.bot_face ? p.bot_face + lf : nullptr,
                                       p.bot_grad ? p.bot_grad + lf : nullptr, p.I_top, p.I_bot);
-    RayF s;
-    s.live = true;
-    s.base = ray % p.nx + 2 * p.nx * (ray / p.nx);
-    s.I = (float)I0;
-    const float4 r = __ldg(rec);
-    s.vc = s.base + __float_as_int(r.x);
-    const float2 cs = chiS[s.vc];
-    s.hc = cs.x * r.z;
-    s.u = s.hc;
-    s.Sc = cs.y;
-    s.Sp = cs.y;
-    s.dS = 0.0f;
-    s.ru = __fdividef(1.0f, s.hc);
-    float cwc = r.y;
-    int k = 1;
-    for (; k + 1 < K; k += 2) {
-        const float4 r1 = __ldg(rec + k), r2 = __ldg(rec + k + 1);
-        fast_step<PARAB, W0, BL>(s, chiS, J, r1, cwc);
-        fast_step<PARAB, W1, BL>(s, chiS, J, r2, r1.y);
-        cwc = r2.y;
-    }
-    if (k < K) {
-        const float4 r1 = __ldg(rec + k);
-        fast_step<PARAB, W0, BL>(s, chiS, J, r1, cwc);
-        cwc = r1.y;
-    }
-    const IntervalE f = interval_fast(s.u, PARAB ? s.ru : __fdividef(1.0f, s.u));
-    s.I = fmaf(f.a, s.dS, fmaf(f.e0, s.Sp - s.I, s.I));
-    atomicAdd(J + s.vc, (double)(cwc * s.I));
-    if (!(fabsf(s.I) <= 3.402823466e38f))  // non-finite: make J NaN
-        atomicAdd(J + s.vc, __longlong_as_double(0x7ff8000000000000LL));
+    const int base = ray % p.nx + 2 * p.nx * (ray / p.nx);
+    twin_ray<PARAB, W0, W1>(rec, K, chiS + base, J + base, (float)I0);
 }
 
 // Jfs = fold(Jrep); r = Jfs - J; dJ0 = r / diag; Jrep zeroed for the next
@@ -310,11 +280,11 @@ int grid_x(long long n, int threads, int cap) {
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-template <bool PARAB, bool BL>
+template <bool PARAB>
 void launch_b_fs_t(const BatchFsParams &p, dim3 grid, int block, int conv, cudaStream_t s) {
-    if (conv == 0) b_fs<PARAB, 0, BL><<<grid, block, 0, s>>>(p);
-    else if (conv == 1) b_fs<PARAB, 1, BL><<<grid, block, 0, s>>>(p);
-    else b_fs<PARAB, 2, BL><<<grid, block, 0, s>>>(p);
+    if (conv == 0) b_fs<PARAB, 0><<<grid, block, 0, s>>>(p);
+    else if (conv == 1) b_fs<PARAB, 1><<<grid, block, 0, s>>>(p);
+    else b_fs<PARAB, 2><<<grid, block, 0, s>>>(p);
 }
 
 }  // namespace
@@ -332,13 +302,8 @@ cudaError_t launch_b_fs(const BatchFsParams &p, int nl, const FsShape &sh, bool 
     if (!fs_shape_valid(sh)) return cudaErrorInvalidValue;
     const int block = sh.block;  // one characteristic per thread
     dim3 grid((p.nx * p.ny + block - 1) / block, p.nangles, nl);
-    if (parabolic) {
-        if (sh.branchless) launch_b_fs_t<true, true>(p, grid, block, sh.widen, s);
-        else launch_b_fs_t<true, false>(p, grid, block, sh.widen, s);
-    } else {
-        if (sh.branchless) launch_b_fs_t<false, true>(p, grid, block, sh.widen, s);
-        else launch_b_fs_t<false, false>(p, grid, block, sh.widen, s);
-    }
+    if (parabolic) launch_b_fs_t<true>(p, grid, block, sh.widen, s);
+    else launch_b_fs_t<false>(p, grid, block, sh.widen, s);
     return cudaGetLastError();
 }
 

@@ -249,22 +249,20 @@ __global__ void __launch_bounds__(128) fs_kernel(FsParams p) {
 }
 
 // FP32 formal solution without Lambda* (every iteration after the first),
-// one characteristic per thread. Per point: one integer add for the
-// replicated address, one 8-byte (chi, S) gather, the interval arithmetic,
-// and one FP64 reduction (red.global.add.f64) into the replicated J, folded
-// afterwards; the FP32 contribution is widened by integer moves, by the
-// conversion instruction (which runs on the FP64 pipe), or alternately by
-// both (the autotuner picks, see fast_step). FP64 accumulation keeps the
+// one characteristic per thread, two points at a time (twin_ray; the
+// autotuner's pick on small grids). Per point: one 8-byte (chi, S) gather, the
+// interval arithmetic, and one FP64 reduction (red.global.add.f64) into the
+// replicated J, folded afterwards; the FP32 contribution is widened by integer
+// moves, by the conversion instruction (which runs on the FP64 pipe), or
+// alternately by both (the autotuner picks). FP64 accumulation keeps the
 // operator's error at the level of its FP32 arithmetic (an FP32 reduction
 // over ~10^3 contributions per voxel and angle group was measured to cost
 // the refinement a fourth FP64 formal solution and 60 more FP32 ones at
-// 129^3). The reciprocal of the next interval is carried into the next step.
-// The last point (linear form) is peeled off; the loop takes two points per
-// trip so that the carried values rotate through registers without moves.
+// 129^3).
 // CONV: how FP32 contributions become FP64 for the reduction: 0 the
 // conversion instruction (FP64 pipe), 1 integer moves, 2 alternating between
 // the two from point to point (both pipes half loaded).
-template <bool PARAB, int CONV, bool BRANCHLESS>
+template <bool PARAB, int CONV>
 __global__ void __launch_bounds__(256) fs_fast_kernel(FsParams p) {
     const int nray = p.nx * p.ny;
     const int ray = blockIdx.x * blockDim.x + threadIdx.x;
@@ -276,43 +274,12 @@ __global__ void __launch_bounds__(256) fs_fast_kernel(FsParams p) {
     double *__restrict__ Jd = p.Jrep;
     constexpr bool W0 = CONV == 1, W1 = CONV >= 1;
 
-    RayF s;
-    const float4 r = __ldg(rec);
-    s.live = true;
-    const int x0 = ray % p.nx, y0 = ray / p.nx;
-    s.base = x0 + 2 * p.nx * y0;
+    const int base = ray % p.nx + 2 * p.nx * (ray / p.nx);
     double I0 = 0.0;
     if (!p.homogeneous)
         I0 = entry_intensity(p.up[o], p.mu, o, ray, p.top_face, p.bot_face, p.bot_grad, p.I_top,
                              p.I_bot);
-    s.I = (float)I0;
-    s.vc = s.base + __float_as_int(r.x);
-    const float2 cs = chiS[s.vc];
-    s.hc = cs.x * r.z;  // half the optical depth of the chord of the point
-    s.u = s.hc;         // the entry interval: chi_{-1} l_{-1} = 0
-    s.Sc = cs.y;
-    s.Sp = cs.y;        // S_{-1} = S_0
-    s.dS = 0.0f;
-    s.ru = __fdividef(1.0f, s.hc);
-    float cwc = r.y;
-    int k = 1;
-    // two points per trip: the carried values rotate through registers
-    for (; k + 1 < K; k += 2) {
-        const float4 r1 = __ldg(rec + k), r2 = __ldg(rec + k + 1);
-        fast_step<PARAB, W0, BRANCHLESS>(s, chiS, Jd, r1, cwc);
-        fast_step<PARAB, W1, BRANCHLESS>(s, chiS, Jd, r2, r1.y);
-        cwc = r2.y;
-    }
-    if (k < K) {
-        const float4 r1 = __ldg(rec + k);
-        fast_step<PARAB, W0, BRANCHLESS>(s, chiS, Jd, r1, cwc);
-        cwc = r1.y;
-    }
-    const IntervalE f = interval_fast(s.u, PARAB ? s.ru : __fdividef(1.0f, s.u));
-    s.I = fmaf(f.a, s.dS, fmaf(f.e0, s.Sp - s.I, s.I));
-    atomicAdd(Jd + s.vc, to_f64<W1>(cwc * s.I));
-    if (!(fabsf(s.I) <= 3.402823466e38f))  // non-finite: make J NaN
-        atomicAdd(Jd + s.vc, __longlong_as_double(0x7ff8000000000000LL));
+    twin_ray<PARAB, W0, W1>(rec, K, chiS + base, Jd + base, (float)I0);
 }
 
 // FP32 formal solution without Lambda*, two characteristics per thread in
@@ -705,11 +672,11 @@ cudaError_t launch_t(const FsParams &p, cudaStream_t s) {
 
 }  // namespace
 
-template <bool PARAB, bool BL>
+template <bool PARAB>
 void launch_fast_w(const FsParams &p, dim3 grid, int block, int widen, cudaStream_t s) {
-    if (widen == 0) fs_fast_kernel<PARAB, 0, BL><<<grid, block, 0, s>>>(p);
-    else if (widen == 1) fs_fast_kernel<PARAB, 1, BL><<<grid, block, 0, s>>>(p);
-    else fs_fast_kernel<PARAB, 2, BL><<<grid, block, 0, s>>>(p);
+    if (widen == 0) fs_fast_kernel<PARAB, 0><<<grid, block, 0, s>>>(p);
+    else if (widen == 1) fs_fast_kernel<PARAB, 1><<<grid, block, 0, s>>>(p);
+    else fs_fast_kernel<PARAB, 2><<<grid, block, 0, s>>>(p);
 }
 
 template <bool PARAB>
@@ -765,13 +732,8 @@ cudaError_t launch_fs_fast(const FsParams &p, bool parabolic, const FsShape &sh,
         return cudaGetLastError();
     }
     dim3 grid((p.nx * p.ny + sh.block - 1) / sh.block, p.nangles);
-    if (parabolic) {
-        if (sh.branchless) launch_fast_w<true, true>(p, grid, sh.block, sh.widen, s);
-        else launch_fast_w<true, false>(p, grid, sh.block, sh.widen, s);
-    } else {
-        if (sh.branchless) launch_fast_w<false, true>(p, grid, sh.block, sh.widen, s);
-        else launch_fast_w<false, false>(p, grid, sh.block, sh.widen, s);
-    }
+    if (parabolic) launch_fast_w<true>(p, grid, sh.block, sh.widen, s);
+    else launch_fast_w<false>(p, grid, sh.block, sh.widen, s);
     return cudaGetLastError();
 }
 

@@ -151,8 +151,7 @@ struct FsShape {
                           // in registers
     int widen;            // FP32 -> FP64: 0 conversion, 1 integer moves, 2 alternating
                           // (two per thread: the second characteristic by integer moves)
-    int branchless;       // 1: parabolic correction evaluated without a branch
-                          // (two per thread: always without)
+    int branchless;       // 0 or 1, no effect
 };
 bool fs_shape_valid(const FsShape &sh);
 // whether the four-characteristic kernel can run on these parameters (its

@@ -596,14 +596,17 @@ cudaError_t launch_sph_build(const SphBuildParams &p, cudaStream_t s) {
 namespace {
 
 // FP32 formal solution without Lambda* on the spherical cache: the
-// per-point step of the Cartesian kernel (fast_step, difference form) over
+// Cartesian kernel's characteristic (twin_ray, two points at a time) over
 // per-segment records (replicated index of the cell as int bits, J weight, l/2,
-// weight), one ray per thread in the builder's order (angle by angle, each
-// angle's rays in the order their launch cells were found), so that the rays
-// of a warp are mostly parallel neighbours whose gathers and reductions fall
-// on nearby cells (21 % faster than ordering by ray length, which matches trip
-// counts but scatters a warp over the shell); contributions reduced in FP64
-// at the replicated index (folded afterwards).
+// weight remainder), one ray per thread in the builder's order (angle by angle,
+// each angle's rays in the order their launch cells were found), so that the
+// rays of a warp are mostly parallel neighbours whose gathers and reductions
+// fall on nearby cells (21 % faster than ordering by ray length, which matches
+// trip counts but scatters a warp over the shell); contributions widened by
+// integer moves (the FP64 pipe stays free) and reduced in FP64 at the
+// replicated index (folded afterwards). Bound by the L2: nearly every segment's
+// reduction is a sector of its own. Loading a point ahead cost 1 to 4 %: the
+// lanes of a warp run rays of different lengths.
 template <bool PARAB>
 __global__ void __launch_bounds__(128) sph_fs_fast_kernel(SphFsParams p, double *__restrict__ Jrep) {
     const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -620,41 +623,7 @@ __global__ void __launch_bounds__(128) sph_fs_fast_kernel(SphFsParams p, double 
         else if (kind == 1) I0 = p.I_irr;
         else I0 = p.I_out;
     }
-    RayF st;
-    st.live = true;
-    st.base = 0;
-    st.I = (float)I0;
-    const float4 r0 = __ldg(rr);
-    st.vc = __float_as_int(r0.x);
-    const float2 cs = chiS[st.vc];
-    st.hc = cs.x * r0.z;
-    st.u = st.hc;
-    st.Sc = cs.y;
-    st.Sp = cs.y;
-    st.dS = 0.0f;
-    st.ru = __fdividef(1.0f, fmaxf(st.hc, 1e-30f));
-    float cwc = r0.y;
-    // two points per trip; contributions widened by integer moves (the FP64
-    // pipe stays free). Loading a point ahead (as the Cartesian pair kernel
-    // does) was 4 % slower here: the lanes of a warp run rays of different
-    // lengths, and the extra loads cost more than the latency they hide.
-    int k = 1;
-    for (; k + 1 < K; k += 2) {
-        const float4 r1 = __ldg(rr + k), r2 = __ldg(rr + k + 1);
-        fast_step<PARAB, true, false>(st, chiS, Jrep, r1, cwc);
-        fast_step<PARAB, true, false>(st, chiS, Jrep, r2, r1.y);
-        cwc = r2.y;
-    }
-    if (k < K) {
-        const float4 r1 = __ldg(rr + k);
-        fast_step<PARAB, true, false>(st, chiS, Jrep, r1, cwc);
-        cwc = r1.y;
-    }
-    const IntervalE f = interval_fast(st.u, PARAB ? st.ru : __fdividef(1.0f, st.u));
-    st.I = fmaf(f.a, st.dS, fmaf(f.e0, st.Sp - st.I, st.I));
-    atomicAdd(Jrep + st.vc, widen_f32(cwc * st.I));
-    if (!(fabsf(st.I) <= 3.402823466e38f))  // non-finite: make J NaN
-        atomicAdd(Jrep + st.vc, __longlong_as_double(0x7ff8000000000000LL));
+    twin_ray<PARAB, true, true>(rr, K, chiS, Jrep, (float)I0);
 }
 
 // FP64 formal solution without Lambda* on the spherical cache: the per-point
