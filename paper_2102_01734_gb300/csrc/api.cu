@@ -1760,6 +1760,27 @@ rt3d_status line_iteration(rt3d_grid *g, const FsParams &fp, bool fp64,
     return RT3D_OK;
 }
 
+// While it lives, formal solutions without Lambda* fold into the caller's J
+// (device memory, aligned): the copy of the grid's J is left out. J may be one
+// of the call's inputs, or hold its boundary faces: the fold writes it after
+// everything has been read, except while the shape is being tuned (one fold per
+// candidate), where the grid's own J is used.
+struct DirectJ {
+    rt3d_grid *g;
+    double *own;
+    DirectJ(rt3d_grid *grid, double *J) : g(grid), own(grid->Jfs) {
+        const bool tunes = !g->sph && !g->fs64 && g->fs_shape.block == 0;
+        if (J && !tunes && (reinterpret_cast<uintptr_t>(J) & 7) == 0) {
+            cudaPointerAttributes at;
+            if (cudaPointerGetAttributes(&at, J) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                ptr_kind(J) == 1)
+                g->Jfs = J;
+            else cudaGetLastError();
+        }
+    }
+    ~DirectJ() { g->Jfs = own; }
+};
+
 }  // namespace
 
 void rt3d::set_last_error(const char *msg) { g_err = msg; }
@@ -1940,6 +1961,7 @@ rt3d_status rt3d_grid_template(const rt3d_grid *gc, int angle, int *K, int32_t *
 rt3d_status rt3d_formal_solution(rt3d_grid *g, const double *chi, const double *S,
                                  const rt3d_bc *bc, double *J_out, double *lstar_out) {
     if (!g || !chi || !S || !J_out) return fail(RT3D_EINVAL, "NULL argument");
+    DirectJ direct(g, lstar_out ? nullptr : J_out);
     const size_t N = (size_t)g->N;
     const double *dchi = nullptr, *dS = nullptr;
     TRY(stage_in(g, chi, N, g->chi, &dchi));
@@ -1957,6 +1979,7 @@ rt3d_status rt3d_formal_solution(rt3d_grid *g, const double *chi, const double *
 rt3d_status rt3d_formal_solution_ff(rt3d_grid *g, const double *chi, const double *S,
                                     const rt3d_bc *bc, double *J_out) {
     if (!g || !chi || !S || !J_out) return fail(RT3D_EINVAL, "NULL argument");
+    DirectJ direct(g, J_out);
     const size_t N = (size_t)g->N;
     const double *dchi = nullptr, *dS = nullptr;
     TRY(stage_in(g, chi, N, g->chi, &dchi));
