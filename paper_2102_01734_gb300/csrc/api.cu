@@ -135,6 +135,7 @@ struct rt3d_grid {
     // the four-characteristic kernel's, x and y exchanged (allocated on first use)
     float4 *pairs_t = nullptr;
     double *Jrep_t = nullptr;
+    double *band_t = nullptr;  // [28 N], with Lambda*; zero between formal solutions
     FsShape fs_shape{0, 0, 0, 0};  // block 0: not chosen yet
     float fs_tune_ms[RT3D_FS_TUNE_SHAPES] = {};  // last tuning: time of each shape
     void *a = nullptr;  // 26 OS off-diagonal planes, os_coef_index layout (f64 in FP64 mode, f32 otherwise)
@@ -557,6 +558,31 @@ rt3d_status run_fs_sph(rt3d_grid *g, const FsParams &base, const void *chiS, int
     return RT3D_OK;
 }
 
+// Whether the four-characteristic kernel builds Lambda* on this grid, with its
+// buffers set up if so (320 bytes a voxel; taken once, within an eighth of the
+// free device memory: where they do not fit, the one-characteristic kernel runs).
+bool lstar_quad(rt3d_grid *g, FsParams *p) {
+    if (g->N > (1LL << 25) || !lstar_quad_applicable(*p)) return false;
+    if (!g->band_t) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        size_t free_b = 0, total_b = 0;
+        if (cudaStreamIsCapturing(g->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+            cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+            320 * (size_t)g->N > free_b / 8) {
+            cudaGetLastError();
+            return false;
+        }
+        double *q = nullptr;
+        const size_t n = 28 * (size_t)g->N;
+        if (quad_setup(g, p) != RT3D_OK || g->alloc(&q, n) != RT3D_OK) return false;
+        if (cudaMemsetAsync(q, 0, sizeof(double) * n, g->stream) != cudaSuccess) return false;
+        g->band_t = q;
+    }
+    if (quad_setup(g, p) != RT3D_OK) return false;
+    p->band_t = g->band_t;
+    return true;
+}
+
 // One formal solution of the packed (chi, S) of the given precision into
 // g->Jfs (zeroed here); Lambda* into g->lstar when requested.
 rt3d_status run_fs(rt3d_grid *g, const FsParams &base, bool fp64, bool with_lstar) {
@@ -573,11 +599,13 @@ rt3d_status run_fs(rt3d_grid *g, const FsParams &base, bool fp64, bool with_lsta
         if (g->fs_shape.block == 0) TRY(fs_tune(g, p));
         if (g->fs_shape.rays_per_thread == 4) TRY(quad_setup(g, &p));
     }
+    const bool lquad = with_lstar && !fp64 && lstar_quad(g, &p);
     if (!fast) CK(cudaMemsetAsync(g->Jfs, 0, sizeof(double) * g->N, g->stream));
     if (with_lstar) CK(cudaMemsetAsync(g->lstar, 0, sizeof(double) * 27 * g->N, g->stream));
     TRY(collect_events(g));
     CK(cudaEventRecord(g->ev0, g->stream));
-    if (fast && fp64) CK(launch_fs64_fast(p, g->parab, g->stream));
+    if (lquad) CK(launch_fs_lstar_quad(p, g->parab, g->stream));
+    else if (fast && fp64) CK(launch_fs64_fast(p, g->parab, g->stream));
     else if (fast) CK(launch_fs_fast(p, g->parab, g->fs_shape, g->stream));
     else CK(launch_fs(p, fp64, g->parab, with_lstar, g->stream));
     CK(cudaEventRecord(g->ev1, g->stream));

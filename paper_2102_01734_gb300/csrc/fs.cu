@@ -478,6 +478,279 @@ __global__ void __launch_bounds__(256, 3) fs_quad_kernel(FsParams p) {
     if (rtop >= 3 && !(fabsf(I1.y) <= 3.402823466e38f)) atomicAdd(j + 3 * rowp, nan);
 }
 
+// FP32 formal solution with Lambda*, four characteristics a thread as above.
+// With one characteristic a thread (fs_kernel) the L2's reduction rate is the
+// bound: J and four to five window entries a segment, 81 % of the rate at 65 x 65
+// x 257. Three of the entries follow the axis of the rows: the voxel itself and,
+// where the step before or after is along that axis, the neighbour up or down a
+// row. Their sums (and J's) ride along in registers, move with the rows and are
+// reduced when a voxel is left; the other entries are reduced at once. The
+// voxel's own entry, by far the largest, carries what its sum loses by rounding.
+// Angles that step along x more run on arrays with x and y exchanged (band_t: the
+// 27 planes and J), added to the others afterwards (band_merge_kernel, 0.16 ms at
+// 97^3). 154 registers: six blocks of 64 a SM without spills; four blocks of 128
+// spill and are no faster. With both kernels and 512 angles: 65 x 65 x 257 27.4 ->
+// 22.5 ms, 97^3 21.2 -> 17.2 ms; L2 reductions at 61 %, issue at 52 %, neither
+// saturated. Error of Lambda* against 64 bits at 65^3: 6.83e-9 -> 6.80e-9 (interval
+// functions from the 9-term series, alpha without cancellation: with the
+// polynomials of the kernel above and e0 - a it was 7.6e-9).
+template <bool PARAB>
+__global__ void __launch_bounds__(64, 6) fs_lstar_quad_kernel(FsParams p) {
+    const int o = p.order4[blockIdx.y];
+    const bool tr = p.swap[o];
+    const int nm = tr ? p.ny : p.nx, nd = tr ? p.nx : p.ny;
+    const int nlive = nm * ((nd + 3) >> 2);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t - (threadIdx.x & 31) >= nlive) return;  // the whole warp is past the face
+    const int tt = min(t, nlive - 1);
+    const int K = p.tlen[o];
+    const float4 *__restrict__ rec = p.rec4 + p.toff[o];
+    const uint32_t *__restrict__ code = p.code + p.toff[o];
+    const unsigned long long *__restrict__ win =
+        reinterpret_cast<const unsigned long long *>(p.win + p.toff[o]);
+    const int m0 = tt % nm, d0 = 4 * (tt / nm);
+    const int rowp = 2 * nm;
+    const float4 *__restrict__ P = (tr ? p.pairs_t : p.pairs) + m0 + rowp * d0;
+    const unsigned row2 = d0 + 2 < nd ? 2 * rowp : 0;
+    const unsigned N = (unsigned)(p.nx * p.ny * p.nz);  // 27 N < 2^31
+    double *__restrict__ band = tr ? p.band_t : p.lstar;
+    double *__restrict__ Jd = tr ? p.band_t + 27ull * N : p.J;
+    const int rtop = t < nlive ? min(3, nd - 1 - d0) : -1;
+    // plane of the neighbour one row up (in the planes' own x, y order)
+    const unsigned up_plane = 13u + (tr ? 1u : 3u), down_plane = 26u - up_plane;
+
+    float Iv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (!p.homogeneous) {
+        const bool up = p.up[o];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (d0 + r < nd) {
+                const int f = tr ? d0 + r + p.nx * m0 : m0 + p.nx * (d0 + r);
+                Iv[r] = (float)entry_intensity(up, p.mu, o, f, p.top_face, p.bot_face, p.bot_grad,
+                                               p.I_top, p.I_bot);
+            }
+    }
+    RayN s[2];
+    float2 ring[2][kWin];
+#pragma unroll
+    for (int i = 0; i < kWin; ++i) ring[0][i] = ring[1][i] = pk1(0.0f);
+    const float4 r0 = __ldg(rec);
+    {
+        const unsigned v = __float_as_uint(r0.x) & kQuadOffMask;
+        quad_start(s[0], __ldg(P + v), pk(r0.z, r0.w), Iv[0], Iv[1]);
+        quad_start(s[1], __ldg(P + (v + row2)), pk(r0.z, r0.w), Iv[2], Iv[3]);
+    }
+    // sums of the rows' current voxels: J, the voxel's own plane, the planes up
+    // and down; used: which of the last two hold anything since the last flush
+    float2 A[4][2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) A[q][0] = A[q][1] = pk1(0.0f);
+    float2 B[2] = {pk1(0.0f), pk1(0.0f)};  // what A[1] lost by rounding
+    bool used_up = false, used_down = false;
+    unsigned v[4];  // the rows' current voxels
+    auto locate = [&](uint32_t c) {
+        const int x = (int)(c & 0x7ffu), y = (int)((c >> 11) & 0x7ffu);
+        int m = m0 + (tr ? y : x), d = d0 + (tr ? x : y);
+        if (m >= nm) m -= nm;
+        if (d >= nd) d -= nd;
+        const unsigned z = (unsigned)(nd * (int)(c >> 22));
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = m + nm * ((d + r >= nd ? d + r - nd : d + r) + z);
+    };
+    auto row = [](const float2 (&a)[2], int r) {
+        return r == 0 ? a[0].x : (r == 1 ? a[0].y : (r == 2 ? a[1].x : a[1].y));
+    };
+    auto reduce = [&](double *__restrict__ to, float2 a, float2 b) {  // all rows
+        if (rtop >= 0) atomicAdd(to + v[0], widen_f32(a.x));
+        if (rtop >= 1) atomicAdd(to + v[1], widen_f32(a.y));
+        if (rtop >= 2) atomicAdd(to + v[2], widen_f32(b.x));
+        if (rtop >= 3) atomicAdd(to + v[3], widen_f32(b.y));
+    };
+    auto target = [&](int q) -> double * {
+        return q == 0 ? Jd : band + N * (q == 1 ? 13u : (q == 2 ? up_plane : down_plane));
+    };
+    // the contributions of the current point: weight cw, window wc, types of
+    // the moves from the previous point and to the next (2: none along the rows)
+    auto contribute = [&](const WeightsN (&wt)[2], float cw, unsigned long long wc, bool first,
+                          unsigned prev, unsigned next, bool ahead) {
+        const float2 c2 = pk1(cw);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+#pragma unroll
+            for (int i = 0; i < kWin - 1; ++i) ring[j][i] = mul2(wt[j].E, ring[j][i + 1]);
+            if (first) ring[j][7] = add2(ring[j][7], wt[j].al);  // S_{-1} = S_0
+            else ring[j][6] = add2(ring[j][6], wt[j].al);
+            ring[j][7] = add2(ring[j][7], wt[j].be);
+            ring[j][8] = wt[j].ga;
+            A[0][j] = fma2(s[j].I, c2, A[0][j]);
+            const float2 sum = fma2(ring[j][7], c2, A[1][j]);
+            B[j] = add2(B[j], fma2(ring[j][7], c2, sub2(A[1][j], sum)));
+            A[1][j] = sum;
+        }
+        // the next point's entry (zero where ga is)
+        if (ahead) {
+            const unsigned dc = (unsigned)(wc >> 40) & 31u;
+            if (next < 2u) {
+                if (next == 0u) {
+                    A[2][0] = fma2(ring[0][8], c2, A[2][0]);
+                    A[2][1] = fma2(ring[1][8], c2, A[2][1]);
+                    used_up = true;
+                } else {
+                    A[3][0] = fma2(ring[0][8], c2, A[3][0]);
+                    A[3][1] = fma2(ring[1][8], c2, A[3][1]);
+                    used_down = true;
+                }
+            } else if (dc != kWinNone) {
+                reduce(band + N * dc, mul2(ring[0][8], c2), mul2(ring[1][8], c2));
+            }
+        }
+        // the previous point's, then the others as long as the run goes on
+        const unsigned d6 = (unsigned)(wc >> 30) & 31u;
+        if (d6 == kWinNone) return;
+        if (prev == 0u) {  // it came one row up: the voxel it left lies down
+            A[3][0] = fma2(ring[0][6], c2, A[3][0]);
+            A[3][1] = fma2(ring[1][6], c2, A[3][1]);
+            used_down = true;
+        } else if (prev == 1u) {
+            A[2][0] = fma2(ring[0][6], c2, A[2][0]);
+            A[2][1] = fma2(ring[1][6], c2, A[2][1]);
+            used_up = true;
+        } else {
+            reduce(band + N * d6, mul2(ring[0][6], c2), mul2(ring[1][6], c2));
+        }
+#pragma unroll
+        for (int i = 5; i >= 0; --i) {
+            const unsigned dc = (unsigned)(wc >> (5 * i)) & 31u;
+            if (dc == kWinNone) break;
+            reduce(band + N * dc, mul2(ring[0][i], c2), mul2(ring[1][i], c2));
+        }
+    };
+    auto flush = [&]() {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (q == 2 && !used_up) continue;
+            if (q == 3 && !used_down) continue;
+            if (q == 1) {
+                double *to = band + N * 13u;
+                if (rtop >= 0) atomicAdd(to + v[0], widen_f32(A[1][0].x) + widen_f32(B[0].x));
+                if (rtop >= 1) atomicAdd(to + v[1], widen_f32(A[1][0].y) + widen_f32(B[0].y));
+                if (rtop >= 2) atomicAdd(to + v[2], widen_f32(A[1][1].x) + widen_f32(B[1].x));
+                if (rtop >= 3) atomicAdd(to + v[3], widen_f32(A[1][1].y) + widen_f32(B[1].y));
+                B[0] = B[1] = pk1(0.0f);
+            } else {
+                reduce(target(q), A[q][0], A[q][1]);
+            }
+            A[q][0] = A[q][1] = pk1(0.0f);
+        }
+        used_up = used_down = false;
+    };
+
+    locate(__ldg(code));
+    unsigned prev = 2u;
+    float cwc = r0.y;
+    float4 rn = __ldg(rec + 1);
+    const unsigned on = __float_as_uint(rn.x) & kQuadOffMask;
+    float4 c[2] = {__ldg(P + on), __ldg(P + (on + row2))};
+    for (int k = 1; k < K; ++k) {
+        const float4 rq = __ldg(rec + k + 1);
+        const unsigned oq = __float_as_uint(rq.x) & kQuadOffMask;
+        const float4 q[2] = {__ldg(P + oq), __ldg(P + (oq + row2))};
+        const unsigned long long wc = __ldg(win + k - 1);
+        const uint32_t cn = __ldg(code + k);
+        WeightsN wt[2];
+        const bool ahead = quad_advance_w<PARAB>(s, c, pk(rn.z, rn.w), wt);
+        const unsigned next = __float_as_uint(rn.x) >> kQuadOffBits;
+        contribute(wt, cwc, wc, k == 1, prev, next, PARAB && ahead);
+        if (next == 0u) {  // one row up: row 0's voxel leaves
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i == 2 && !used_up) continue;
+                if (i == 3 && !used_down) continue;
+                if (rtop >= 0)
+                    atomicAdd(target(i) + v[0], i == 1 ? widen_f32(A[1][0].x) + widen_f32(B[0].x)
+                                                       : widen_f32(A[i][0].x));
+                A[i][0] = pk(A[i][0].y, A[i][1].x);
+                A[i][1] = pk(A[i][1].y, 0.0f);
+                if (rtop < 3) {  // the last existing row enters a voxel no sum holds
+                    if (rtop == 2) A[i][1].x = 0.0f;
+                    else if (rtop == 1) A[i][0].y = 0.0f;
+                    else A[i][0].x = 0.0f;
+                }
+            }
+            B[0] = pk(B[0].y, B[1].x);
+            B[1] = pk(B[1].y, 0.0f);
+            if (rtop == 2) B[1].x = 0.0f;
+            else if (rtop == 1) B[0].y = 0.0f;
+            else if (rtop == 0) B[0].x = 0.0f;
+        } else if (next == 1u) {  // one row down: the last existing row's voxel leaves
+            const unsigned vt = rtop == 3 ? v[3] : (rtop == 2 ? v[2] : (rtop == 1 ? v[1] : v[0]));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i == 2 && !used_up) continue;
+                if (i == 3 && !used_down) continue;
+                if (rtop >= 0)
+                    atomicAdd(target(i) + vt, i == 1 ? widen_f32(row(A[1], rtop)) + widen_f32(row(B, rtop))
+                                                     : widen_f32(row(A[i], rtop)));
+                A[i][1] = pk(A[i][0].y, A[i][1].x);
+                A[i][0] = pk(0.0f, A[i][0].x);
+            }
+            B[1] = pk(B[0].y, B[1].x);
+            B[0] = pk(0.0f, B[0].x);
+        } else {
+            flush();
+        }
+        prev = next;
+        locate(cn);
+        cwc = rn.y;
+        rn = rq;
+        c[0] = q[0];
+        c[1] = q[1];
+    }
+    WeightsN wt[2];
+    quad_last_w(s[0], wt[0]);
+    quad_last_w(s[1], wt[1]);
+    contribute(wt, cwc, __ldg(win + K - 1), K == 1, prev, 2u, false);
+    flush();
+    // a non-finite intensity persists along the recurrence: make J NaN
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    if (rtop >= 0 && !(fabsf(s[0].I.x) <= 3.402823466e38f)) atomicAdd(Jd + v[0], nan);
+    if (rtop >= 1 && !(fabsf(s[0].I.y) <= 3.402823466e38f)) atomicAdd(Jd + v[1], nan);
+    if (rtop >= 2 && !(fabsf(s[1].I.x) <= 3.402823466e38f)) atomicAdd(Jd + v[2], nan);
+    if (rtop >= 3 && !(fabsf(s[1].I.y) <= 3.402823466e38f)) atomicAdd(Jd + v[3], nan);
+}
+
+// The exchanged planes (grid z = 27 nz + z: the plane, J last, and the layer)
+// transposed onto the others, 32 x 32 at a time, and zeroed for the next call.
+__global__ void __launch_bounds__(256) band_merge_kernel(int nx, int ny, int nz, double *__restrict__ band_t,
+                                                         double *__restrict__ lstar,
+                                                         double *__restrict__ J) {
+    __shared__ double tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+    const long long n = (long long)nx * ny;
+    for (int l = blockIdx.z; l < 28 * nz; l += gridDim.z) {
+        double *__restrict__ from = band_t + n * l + y0 + tx;
+        double *__restrict__ to = (l < 27 * nz ? lstar + n * l : J + n * (l - 27 * nz)) + x0 + tx;
+        double a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // all loads first
+            const int x = x0 + ty + 8 * i, y = y0 + ty + 8 * i;
+            a[i] = x < nx && y0 + tx < ny ? from[(long long)ny * x] : 0.0;
+            b[i] = y < ny && x0 + tx < nx ? to[(long long)nx * y] : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tile[ty + 8 * i][tx] = a[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int x = x0 + ty + 8 * i, y = y0 + ty + 8 * i;
+            if (x < nx && y0 + tx < ny) from[(long long)ny * x] = 0.0;
+            if (y < ny && x0 + tx < nx) to[(long long)nx * y] = b[i] + tile[tx][ty + 8 * i];
+        }
+        __syncthreads();
+    }
+}
+
 // Records of the four-characteristic kernel: (offset | step type << 29,
 // J weight, l/2, l/2), offsets with x and y exchanged for the angles that swap
 // them, the step type of the move from the previous point: 0 one row up, 1 one
@@ -692,6 +965,37 @@ void launch_pair_w(const FsParams &p, dim3 grid, int block, int widen, cudaStrea
     else fs_pair_kernel<PARAB, 2><<<grid, block, 0, s>>>(p);
 }
 
+// groups of four characteristics of one angle, the larger of the two splits
+static int lane_count(const FsParams &p) {
+    return std::max(p.nx * ((p.ny + 3) / 4), p.ny * ((p.nx + 3) / 4));
+}
+
+cudaError_t launch_fs_lstar_quad(const FsParams &p, bool parabolic, cudaStream_t s) {
+    const int rows = 2 * p.ny * p.nz;
+    const float2 *chiS = static_cast<const float2 *>(p.chiS);
+    pair_pack_kernel<<<rows < 65536 ? rows : 65536, 256, 0, s>>>(p.nx, p.ny, p.nz, chiS, p.pairs);
+    pair_pack_t_kernel<<<dim3((2 * p.nx + 31) / 32, (2 * p.ny + 31) / 32, p.nz), 256, 0, s>>>(
+        p.nx, p.ny, chiS, p.pairs_t);
+    const dim3 grid((lane_count(p) + 63) / 64, p.nangles);
+    if (parabolic) fs_lstar_quad_kernel<true><<<grid, 64, 0, s>>>(p);
+    else fs_lstar_quad_kernel<false><<<grid, 64, 0, s>>>(p);
+    band_merge_kernel<<<dim3((p.nx + 31) / 32, (p.ny + 31) / 32, std::min(28 * p.nz, 65535)), 256, 0, s>>>(
+        p.nx, p.ny, p.nz, p.band_t, p.lstar, p.J);
+    return cudaGetLastError();
+}
+
+// Below about 3.5 waves of groups (384 of them resident per SM) the coarser
+// split leaves the last wave too empty: at 65^3 voxels the kernel takes 1.60 ms
+// against 1.56 with one characteristic a thread for 141,000 groups (8 x 16
+// angles), 3.13 against 3.47 for 318,000 (12 x 24) and 5.4 against 6.3 for 566,000
+// (16 x 32); at 33^3 1.26 against 1.27 for 152,000. Sides of one or two
+// voxels are left out: there the neighbours up and down a row coincide.
+bool lstar_quad_applicable(const FsParams &p) {
+    const long long groups = (long long)lane_count(p) * p.nangles;
+    return quad_applicable(p) && std::min(p.nx, p.ny) >= 4 && 27LL * p.nx * p.ny * p.nz < (1LL << 31) &&
+           2 * groups >= 7LL * 384 * device_sm_count();
+}
+
 bool quad_applicable(const FsParams &p) {
     return p.rec4 != nullptr && 4LL * p.nx * p.ny * p.nz <= (long long)kQuadOffMask;
 }
@@ -719,8 +1023,7 @@ cudaError_t launch_fs_fast(const FsParams &p, bool parabolic, const FsShape &sh,
         if (sh.rays_per_thread == 4) {
             pair_pack_t_kernel<<<dim3((2 * p.nx + 31) / 32, (2 * p.ny + 31) / 32, p.nz), 256, 0, s>>>(
                 p.nx, p.ny, static_cast<const float2 *>(p.chiS), p.pairs_t);
-            const int nlanes = std::max(p.nx * ((p.ny + 3) / 4), p.ny * ((p.nx + 3) / 4));
-            dim3 grid((nlanes + sh.block - 1) / sh.block, p.nangles);
+            dim3 grid((lane_count(p) + sh.block - 1) / sh.block, p.nangles);
             if (parabolic) launch_quad_w<true>(p, grid, sh.block, sh.widen, s);
             else launch_quad_w<false>(p, grid, sh.block, sh.widen, s);
             return cudaGetLastError();

@@ -332,6 +332,128 @@ __device__ __forceinline__ void quad_start(RayN &s, const float4 &c, float2 hl, 
     s.nD = pk1(0.0f);
 }
 
+// ---- The same with the weights of Lambda*'s window ----
+// E = e^-u, al, be and ga: the derivatives of I_k by I_{k-1}, S_{k-1}, S_k and
+// S_{k+1} over its own interval.
+struct WeightsN {
+    float2 E, al, be, ga;
+};
+// Interval functions with E and al of the linear form: below 1 from the 9-term
+// series of p(u), as in the one-characteristic kernel with Lambda*, and e0 - a in
+// the form u ((1 + b)/2 - a), which does not cancel.
+__device__ __forceinline__ IntervalN2 interval_thin_w(float2 u, WeightsN &w) {
+    float2 np = pk1((float)(-2.0 / 39916800.0));  // -p(u), the Taylor polynomial
+    np = fma2(np, u, pk1((float)(2.0 / 3628800.0)));
+    np = fma2(np, u, pk1((float)(-2.0 / 362880.0)));
+    np = fma2(np, u, pk1((float)(2.0 / 40320.0)));
+    np = fma2(np, u, pk1((float)(-2.0 / 5040.0)));
+    np = fma2(np, u, pk1((float)(2.0 / 720.0)));
+    np = fma2(np, u, pk1((float)(-2.0 / 120.0)));
+    np = fma2(np, u, pk1((float)(2.0 / 24.0)));
+    np = fma2(np, u, pk1((float)(-2.0 / 6.0)));
+    const float2 nb = mul2(u, np);
+    const float2 nhu = mul2(u, pk1(-0.5f));
+    IntervalN2 r;
+    r.na = fma2(nhu, nb, nhu);
+    r.e0 = fma2(u, r.na, u);
+    r.d = sub2(nb, r.na);
+    w.E = sub2(pk1(1.0f), r.e0);
+    w.al = mul2(u, add2(fma2(nb, pk1(-0.5f), pk1(0.5f)), r.na));
+    return r;
+}
+__device__ __forceinline__ IntervalN2 interval_thick_w(float2 u, WeightsN &w) {
+    const float2 t = mul2(u, pk1(-1.4426950408889634f));
+    w.E = pk(ex2_approx(t.x), ex2_approx(t.y));
+    const float2 ru = pk(rcp_approx(u.x), rcp_approx(u.y));
+    IntervalN2 r;
+    r.e0 = sub2(pk1(1.0f), w.E);
+    r.na = fma2(r.e0, ru, pk1(-1.0f));
+    r.d = pk1(0.0f);
+    w.al = sub2(mul2(r.e0, ru), w.E);
+    return r;
+}
+// f, w: the thin form's; the thick form's where u >= 1
+__device__ __forceinline__ IntervalN2 select_w(float2 u, IntervalN2 f, WeightsN &w) {
+    WeightsN h;
+    const IntervalN2 e = interval_thick_w(u, h);
+    const bool x = u.x < 1.0f, y = u.y < 1.0f;
+    IntervalN2 r;
+    r.e0 = pk(x ? f.e0.x : e.e0.x, y ? f.e0.y : e.e0.y);
+    r.na = pk(x ? f.na.x : e.na.x, y ? f.na.y : e.na.y);
+    r.d = pk(x ? f.d.x : 0.0f, y ? f.d.y : 0.0f);
+    w.E = pk(x ? w.E.x : h.E.x, y ? w.E.y : h.E.y);
+    w.al = pk(x ? w.al.x : h.al.x, y ? w.al.y : h.al.y);
+    return r;
+}
+// quad_advance with the weights; false when all intervals are thick (ga = 0).
+template <bool PARAB>
+__device__ __forceinline__ bool quad_advance_w(RayN (&s)[2], const float4 (&c)[2], float2 hl,
+                                               WeightsN (&wt)[2]) {
+    float2 hn[2], Sn[2], nDn[2], w[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        hn[j] = mul2(pk(c[j].x, c[j].y), hl);
+        Sn[j] = pk(c[j].z, c[j].w);
+        nDn[j] = sub2(s[j].Sc, Sn[j]);
+        w[j] = add2(s[j].hc, hn[j]);
+    }
+    const float lo = fminf(fminf(s[0].u.x, s[0].u.y), fminf(s[1].u.x, s[1].u.y));
+    const bool all_thick = __all_sync(0xffffffffu, lo >= 1.0f);
+    if (all_thick) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const IntervalN2 f = interval_thick_w(s[j].u, wt[j]);
+            wt[j].be = sub2(pk1(0.0f), f.na);
+            wt[j].ga = pk1(0.0f);
+            s[j].I = linear_n(s[j], f);
+        }
+    } else {
+        const float hi = fmaxf(fmaxf(s[0].u.x, s[0].u.y), fmaxf(s[1].u.x, s[1].u.y));
+        const bool all_thin = __all_sync(0xffffffffu, hi < 1.0f);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 u = s[j].u;
+            IntervalN2 f = interval_thin_w(u, wt[j]);
+            if (!all_thin) f = select_w(u, f, wt[j]);
+            float2 In = linear_n(s[j], f);
+            float2 g = pk1(0.0f), qg = pk1(0.0f);  // -f s d and q f s d
+            if (PARAB) {  // as parabola_n
+                const float2 nwf = pk(fminf(-w[j].x, -1e-15f), fminf(-w[j].y, -1e-15f));
+                const float2 nuw = sub2(nwf, u);
+                const float2 nq = mul2(u, pk(rcp_approx(nwf.x), rcp_approx(nwf.y)));
+                const float2 ns = mul2(u, pk(rcp_approx(nuw.x), rcp_approx(nuw.y)));
+                const float2 fw = mul2(pk(__saturatef(fmaf(-2.0f, u.x, 2.0f)),
+                                          __saturatef(fmaf(-2.0f, u.y, 2.0f))),
+                                       pk(__saturatef(fmaf(0.5f, nq.x, 2.0f)),
+                                          __saturatef(fmaf(0.5f, nq.y, 2.0f))));
+                g = mul2(mul2(fw, f.d), ns);
+                qg = mul2(nq, g);
+                In = fma2(g, fma2(nq, nDn[j], s[j].nD), In);
+            }
+            wt[j].al = add2(wt[j].al, g);
+            wt[j].be = sub2(qg, add2(f.na, g));
+            wt[j].ga = sub2(pk1(0.0f), qg);
+            s[j].I = In;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        s[j].u = w[j];
+        s[j].hc = hn[j];
+        s[j].Sp = s[j].Sc;
+        s[j].Sc = Sn[j];
+        s[j].nD = nDn[j];
+    }
+    return !all_thick;
+}
+// The last point's (linear form).
+__device__ __forceinline__ void quad_last_w(RayN &s, WeightsN &w) {
+    const IntervalN2 f = select_w(s.u, interval_thin_w(s.u, w), w);
+    w.be = sub2(pk1(0.0f), f.na);
+    w.ga = pk1(0.0f);
+    s.I = linear_n(s, f);
+}
+
 // ---- One characteristic, two successive points at a time ----
 // Components .x and .y are points k and k + 1 of the same characteristic: all
 // that does not depend on the intensity is evaluated for both in one packed

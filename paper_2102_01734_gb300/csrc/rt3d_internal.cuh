@@ -108,6 +108,8 @@ struct FsParams {
     const int *order4;
     float4 *pairs_t;     // with rec4: [4N] pairs with x and y exchanged
     double *Jrep_t;      // with rec4: [4N] Jrep with x and y exchanged
+    double *band_t;      // with rec4 and lstar: [28 N], the planes and J with x and y
+                         // exchanged (zero between launches)
     double *lstar;     // nullable [27][N], accumulated into
     const double *top_face;  // nullable [ny*nx]
     const double *bot_face;  // nullable [ny*nx]
@@ -157,6 +159,11 @@ bool fs_shape_valid(const FsShape &sh);
 // whether the four-characteristic kernel can run on these parameters (its
 // records exist and the replicated grid's offsets fit in 29 bits)
 bool quad_applicable(const FsParams &p);
+// FP32 formal solution with Lambda*, four characteristics per thread: into p.J
+// and p.lstar (zeroed by the caller); whether it can run on these parameters and
+// fills the device
+bool lstar_quad_applicable(const FsParams &p);
+cudaError_t launch_fs_lstar_quad(const FsParams &p, bool parabolic, cudaStream_t s);
 // the four-characteristic kernel's step records from the template
 cudaError_t launch_quad_rec(const Template &t, int nx, int ny, float4 *rec4, cudaStream_t s);
 // FP32 formal solution without Lambda* into p.Jrep (zero on entry; the fold
