@@ -406,8 +406,8 @@ rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
     // above 2^25 voxels the four-characteristic kernel's 96 bytes a voxel are
     // left to the solver's vectors
-    const bool four = quad_applicable(p) && g->N <= (1LL << 25);
-    if (four) TRY(quad_setup(g, &p));
+    // (nor is it a reason to fail: where its buffers do not fit it is not timed)
+    const bool four = quad_applicable(p) && g->N <= (1LL << 25) && quad_setup(g, &p) == RT3D_OK;
     float best = 0.0f;
     int pick = 0;
     for (int i = -1; i < RT3D_FS_TUNE_SHAPES; ++i) {
