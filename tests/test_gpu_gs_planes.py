@@ -1,8 +1,8 @@
 """The OS sweeps where their split changes: solves whose coefficients stay in
 shared memory (from one block on, the last ones that fit and the first that do
 not), and above them the Gauss-Seidel plane kernel with one block to eight per
-plane, odd and even axes, flat and tall boxes; Jacobi and Gauss-Seidel, both
-precisions."""
+plane, or the Jacobi sweep with less than one block a warp to many, odd and even
+axes, flat and tall boxes; Jacobi and Gauss-Seidel, both precisions."""
 import numpy as np
 import pytest
 
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n", [(4, 4, 1), (5, 4, 2), (6, 37, 3), (33, 70, 9), (4, 6, 130), (64, 64, 38),
                                (65, 65, 65), (68, 65, 71), (130, 5, 600), (65, 80, 70), (70, 300, 18),
-                               (300, 70, 18), (512, 513, 2)])
+                               (300, 70, 18), (512, 513, 2), (5, 5, 521)])
 @pytest.mark.parametrize("fp64", [True, False])
 @pytest.mark.parametrize("gs", [True, False])
 def test_against_oracle(n, fp64, gs):
