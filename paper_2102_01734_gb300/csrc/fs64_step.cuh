@@ -1,8 +1,9 @@
 // FP64 per-point arithmetic of the formal solutions without Lambda*,
 // shared by the Cartesian kernel (fs.cu) and the spherical one (sph.cu). The
-// FP64 pipe is the bound, so everything that can leave it does: branch tests
-// on the high word of non-negative doubles (integer compares), reciprocals
-// seeded in FP32, widening by integer moves. The interval functions follow
+// FP64 pipe is the bound, so everything that can leave it does (an FP64
+// instruction holds its pipe for 64 cycles, in which 64 others issue): branch
+// tests on the high word of non-negative doubles (integer compares), reciprocals,
+// the polynomial's smaller terms, halving, widening by integer moves. The interval functions follow
 // the construction documented at the top of fs.cu (Olson & Kunasz 1987
 // weights; the update in difference form).
 #pragma once
@@ -18,20 +19,62 @@ __device__ __forceinline__ bool hi_below(double x, int b_hi) {
     return (unsigned)__double2hiint(x) < (unsigned)b_hi;
 }
 
-// 1/x for x > 0. Seed: x truncated to FP32 by integer moves (for x and 1/x
-// inside the FP32 normal range: exponent field 897..1148), its FP32
-// reciprocal, widened back; then one third-order Newton-Raphson step
-// r = r0 + r0 (e + e^2), e = 1 - x r0, which takes the seed's relative error
-// (< 2^-21, the hardware approximation's 2^-23 and the truncation) to below 2^-63, so the result is within an ulp or so of 1/x.
-// Outside that range (and for 0, Inf, NaN): IEEE division.
+// a + b = s + t exactly (Knuth)
+__device__ __forceinline__ float sum_exact(float a, float b, float &t) {
+    const float s = a + b, bb = s - a;
+    t = (a - (s - bb)) + (b - bb);
+    return s;
+}
+
+// 1/x for x > 0, without the FP64 pipe. With x = 2^k m, 1 <= m < 2, m is split
+// by integer moves into its first 24 bits, the next 24 and the last 5 (xh, xl,
+// xt); r0 is the FP32 reciprocal of xh. The residual e = 1 - m r0 (|e| < 2^-21) is
+// collected as a pair of FP32 values (eh, el) whose error is below 2^-66, the
+// correction r0 (e + e^2) likewise (the next term, e^3, is below 2^-63), and the
+// sum r0 + correction is formed and rounded in fixed point (units of 2^-60): within
+// 0.52 units in the last place of 1/x. For 0, subnormal, infinite and NaN x and x from
+// 2^1021 on: IEEE division.
 __device__ __forceinline__ double recip64(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x);
-    if (((hi >> 20) & 0x7ffu) - 897u > 251u || (hi >> 31)) return 1.0 / x;
-    const unsigned lo = (unsigned)__double2loint(x);
-    const float xf = __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
-    const double r0 = widen_f32(rcp_approx(xf));
-    const double e = fma(-x, r0, 1.0);
-    return fma(r0, fma(e, e, e), r0);
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned ex = hi >> 20;
+    if (ex - 1u > 2042u) return 1.0 / x;
+    const float xh = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const float xl = (float)(lo & 0x1fffffe0u) * 0x1p-52f, xt = (float)(lo & 31u) * 0x1p-52f;
+    const float r0 = rcp_approx(xh);
+    const float ph = xh * r0, pl = fmaf(xh, r0, -ph);
+    const float q = xl * r0, ql = fmaf(xl, r0, -q);
+    float t1, t2;
+    const float s1 = sum_exact(1.0f - ph, -q, t1);
+    const float eh = sum_exact(s1, -pl, t2);
+    const float el = fmaf(-xt, r0, (t1 + t2) - ql);
+    const float f = fmaf(eh, eh, el);
+    const float ch = r0 * eh, cl = fmaf(r0, f, fmaf(r0, eh, -ch));
+    // r0 2^60, the correction's first 23 bits and the rest
+    const int c1 = __float2int_rn(ch * 0x1p44f);
+    const int c2 = __float2int_rn((fmaf((float)c1, -0x1p-44f, ch) + cl) * 0x1p60f);
+    const long long fix = ((long long)__float2int_rn(r0 * 0x1p24f) << 36) + ((long long)c1 << 16) + c2;
+    // 2^59 <= fix <= 2^60: 53 bits, rounded; 1 carries into the exponent
+    const long long bits = ((fix + 64) >> 7) + (1021LL << 52) - ((long long)((int)ex - 1023) << 52);
+    return __longlong_as_double(bits);
+}
+
+// (h, l) = c + u (h, l) in float-float, |c| > |u h|
+__device__ __forceinline__ void horner_ff(float &h, float &l, float uh, float ul, double c) {
+    const float chi = (float)c, clo = (float)(c - (double)chi);  // folded at compile time
+    const float p = uh * h;
+    const float e = fmaf(uh, l, fmaf(ul, h, fmaf(uh, h, -p)));
+    const float s = chi + p;
+    l = (p - (s - chi)) + (e + clo);
+    h = s;
+}
+// |x| as a pair of FP32 values, x = +-(h + l) to 2^-48 of it, by integer moves;
+// both 0 below 2^-38, for |x| < 2^127.
+__device__ __forceinline__ void split_ff(double x, float &h, float &l) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+    const unsigned ex = hi >> 20;
+    const bool tiny = ex < 985u;
+    h = tiny ? 0.0f : __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
+    l = tiny ? 0.0f : (float)(lo & 0x1fffffffu) * __uint_as_float((ex - 948u) << 23);
 }
 
 // 2^(-j/64), j = 0 .. 63, correctly rounded.
@@ -64,10 +107,10 @@ __device__ __forceinline__ void exp_table(double *tab) {
 // e^-u for 1/2 <= u < 37.5 (Tang's table-driven method): n = nearest integer
 // to 64 u / ln2 (found in FP32; a neighbour of it near a tie only widens r's
 // range), r = u - n ln2/64, |r| <= ln2/128 (1 + 2^-9), e^-r by its Taylor
-// polynomial of degree 5 (truncation r^6/720 < 4e-17), e^-u = 2^-(n div 64)
-// 2^-((n mod 64)/64) e^-r. Eight FP64 operations, about half of the library's
-// exp, whose accuracy over the whole range e^-u does not need here: the caller
-// takes 1 - e^-u.
+// polynomial of degree 5 (truncation r^6/720 < 4e-17; the terms from r^2 on, below
+// 2^-15, in float-float), e^-u = 2^-(n div 64) 2^-((n mod 64)/64) e^-r. Five FP64
+// operations, a third of the library's exp, whose accuracy over the whole range
+// e^-u does not need here: the caller takes 1 - e^-u.
 __device__ __forceinline__ double exp_neg64(double u, const double *tab) {
     const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
     const float uf = __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
@@ -75,21 +118,43 @@ __device__ __forceinline__ double exp_neg64(double u, const double *tab) {
     const int n = __float_as_int(t) - 0x4B400000;
     const double nd = widen_f32(t - 12582912.0f);
     const double r = fma(-nd, kLn2Lo, fma(-nd, kLn2Hi, u));
-    double q = fma(r, -1.0 / 120.0, 1.0 / 24.0);
-    q = fma(r, q, -1.0 / 6.0);
-    q = fma(r, q, 0.5);
-    const double P = fma(r * r, q, -r);  // e^-r - 1
+    float rh, rl;
+    split_ff(r, rh, rl);
+    if (r < 0.0) {
+        rh = -rh;
+        rl = -rl;
+    }
+    float h = fmaf(rh, (float)(-1.0 / 120.0), (float)(1.0 / 24.0)), l = 0.0f;
+    horner_ff(h, l, rh, rl, -1.0 / 6.0);
+    horner_ff(h, l, rh, rl, 0.5);
+    const float p = rh * rh, e = fmaf(rh, 2.0f * rl, fmaf(rh, rh, -p));  // r^2
+    const float gh = p * h, gl = fmaf(e, h, fmaf(p, l, fmaf(p, h, -gh)));
+    const double P = (widen_f32(gl) - r) + widen_f32(gh);  // e^-r - 1
     const double T = tab[n & 63];
     const double E = fma(T, P, T);
     return __hiloint2double(__double2hiint(E) - ((n >> 6) << 20), __double2loint(E));
 }
 
+// The terms of p(u) from degree 3 on, over u^3, for 0 <= u < 1/2, in float-float
+// (degrees 8 and 9 in FP32): together they are below 2^-9 of p, and their error
+// below 2^-46 of themselves. Below 2^-38 only the first counts.
+__device__ __forceinline__ double tail64(double u) {
+    float uh, ul;
+    split_ff(u, uh, ul);
+    float h = fmaf(uh, -3.4475018036590732e-09f, 4.9354831016668725e-08f), l = 0.0f;
+    horner_ff(h, l, uh, ul, -5.507115670485655e-07);
+    horner_ff(h, l, uh, ul, 5.511310234105578e-06);
+    horner_ff(h, l, uh, ul, -4.9603140878306714e-05);
+    horner_ff(h, l, uh, ul, 3.9682539230545495e-04);
+    horner_ff(h, l, uh, ul, -2.777777777429071e-03);
+    return widen_f32(h) + widen_f32(l);
+}
+
 // Interval functions in FP64 (as interval(double)); for u < 1/2 p(u) =
 // e2/u^3 is a degree-9 polynomial fitted to the exact function (least squares
 // in relative error at 300 Chebyshev nodes of [0, 1/2]; FP64 Horner error
-// 1.6e-16 relative, the rounding of its leading coefficient 1/3). The terms of
-// degree 7 to 9 are left out below 2^-6 and those of degree 5 and 6 below 2^-10,
-// where they are under 4e-19 and 2e-18 of the sum. From 37.5 on e^-u is below
+// 1.6e-16 relative, the rounding of its leading coefficient 1/3), its terms from
+// degree 3 on evaluated off the FP64 pipe (tail64). From 37.5 on e^-u is below
 // 2^-54, and e0 = 1 (a NaN u goes there and reaches a through ru). ru = 1/u
 // for u >= 1/2 (carried from the previous step, or computed here if CARRY is
 // false). Returns e0, a, d for the update in difference form.
@@ -100,26 +165,12 @@ template <bool CARRY>
 __device__ __forceinline__ IntervalDE interval64(double u, double ru, const double *tab) {
     IntervalDE r;
     if (hi_below(u, 0x3FE00000)) {
-        double p = -3.4475018036590732e-09;
-        if (hi_below(u, 0x3F900000)) {
-            p = 5.511310234105578e-06;
-        } else {
-            p = fma(p, u, 4.9354831016668725e-08);
-            p = fma(p, u, -5.507115670485655e-07);
-            p = fma(p, u, 5.511310234105578e-06);
-        }
-        if (hi_below(u, 0x3F500000)) {
-            p = 3.9682539230545495e-04;
-        } else {
-            p = fma(p, u, -4.9603140878306714e-05);
-            p = fma(p, u, 3.9682539230545495e-04);
-        }
-        p = fma(p, u, -2.777777777429071e-03);
+        double p = tail64(u);
         p = fma(p, u, 1.6666666666652976e-02);
         p = fma(p, u, -8.333333333333312e-02);
         p = fma(p, u, 3.333333333333333e-01);
         const double b = u * p;
-        const double hu = 0.5 * u;
+        const double hu = __hiloint2double(max(0, __double2hiint(u) - 0x00100000), __double2loint(u));  // u / 2
         const double a = fma(-hu, b, hu);
         r.e0 = fma(-u, a, u);
         r.a = a;

@@ -673,10 +673,9 @@ __global__ void __launch_bounds__(128) sph_fs64_fast_kernel(SphFsParams p, doubl
             const double rw = recip64(w);
             const double q = u * rw;
             if (hi_below(u, 0x3FF00000) && hi_below(q, 0x40100000)) {
-                double fw = 1.0;
-                if (!hi_below(u, 0x3FE00000)) fw = fma(-2.0, u, 2.0);
-                if (!hi_below(q, 0x40000000)) fw *= fma(-0.5, q, 2.0);
-                const double sd = fw * (u * recip64(u + w)) * f.d;
+                double sd = u * recip64(u + w) * f.d;
+                if (!hi_below(u, 0x3FE00000)) sd *= fma(-2.0, u, 2.0);
+                if (!hi_below(q, 0x40000000)) sd *= fma(-0.5, q, 2.0);
                 In = fma(sd, fma(-q, dSn, dS), In);
             }
             ru = rw;

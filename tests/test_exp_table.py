@@ -1,6 +1,8 @@
-"""The table and constants of the FP64 kernels' e^-u, and its error."""
+"""The FP64 kernels' e^-u (its table, constants and error), reciprocal and
+polynomial tail."""
 import os
 import re
+from fractions import Fraction
 
 import mpmath
 import numpy as np
@@ -50,9 +52,49 @@ def test_error_of_exp_neg():
     assert worst < 2.5 * 2.0 ** -53
 
 
-def test_short_polynomials():
-    """What the branches below 2^-6 and 2^-10 leave out of p(u) (leading term
-    1/3) stays below a fiftieth of its last bit."""
-    c = {m: 2.0 / float(mpmath.factorial(m + 3)) for m in range(5, 10)}
-    assert 3 * c[7] * 2.0 ** (-6 * 7) < 2.0 ** -53 / 50
-    assert 3 * c[5] * 2.0 ** (-10 * 5) < 2.0 ** -53 / 50
+def _rd(x):
+    """A fraction rounded to FP32."""
+    return Fraction(float(np.float32(float(x))))
+
+
+def test_reciprocal():
+    """recip64 step by step, each FP32 operation rounded once, from a seed one
+    FP32 unit off either way: at most 0.52 units in the last place."""
+    rng = np.random.default_rng(2)
+    x = np.concatenate([[1.0, np.nextafter(1.0, 2), np.nextafter(2.0, 1), 1.5, 1 + 2.0 ** -24, 2 - 2.0 ** -24],
+                        1 + rng.uniform(0, 1, 2000)])
+    worst = 0.0
+    for i, v in enumerate(x):
+        m = Fraction(float(v))
+        k = int(m * 2 ** 52)
+        xh, xl, xt = Fraction(k >> 29, 2 ** 23), Fraction(k & 0x1fffffe0, 2 ** 52), Fraction(k & 31, 2 ** 52)
+        assert xh + xl + xt == m and _rd(xl) == xl
+        r0 = np.float32(float(1 / xh))
+        r0 = Fraction(float([r0, np.nextafter(r0, np.float32(0)), min(np.nextafter(r0, np.float32(2)), np.float32(1))][i % 3]))
+        ph = _rd(xh * r0)
+        pl = _rd(xh * r0 - ph)
+        q = _rd(xl * r0)
+        ql = _rd(xl * r0 - q)
+        a = _rd(1 - ph)
+        s1 = _rd(a - q)
+        eh = _rd(s1 - pl)
+        el = _rd(_rd(_rd((a - q - s1) + (s1 - pl - eh)) - ql) - xt * r0)
+        f = _rd(eh * eh + el)
+        ch = _rd(r0 * eh)
+        cl = _rd(r0 * f + _rd(r0 * eh - ch))
+        c1 = round(ch * 2 ** 44)
+        c2 = round(_rd(_rd(ch - Fraction(c1, 2 ** 44)) + cl) * 2 ** 60)
+        fix = (int(r0 * 2 ** 24) << 36) + (c1 << 16) + c2
+        assert abs(c1) < 2 ** 23 and abs(c2) < 2 ** 24
+        assert 2 ** 59 <= fix + 64 <= 2 ** 60 + 128
+        worst = max(worst, abs(float(Fraction((fix + 64) >> 7, 2 ** 53) * m - 1)) * 2 ** 53 / float(m) * 1.0)
+    assert worst < 0.52
+
+
+def test_tail_weight():
+    """What tail64 evaluates in float-float is below 2^-9 of p(u) on [0, 1/2], and
+    its terms of degree 8 and 9, in FP32, below 2^-30."""
+    c = {m: 2.0 / float(mpmath.factorial(m + 3)) for m in range(10)}
+    p = 1 / 3 - 0.5 / 12
+    assert sum(c[m] * 0.5 ** m for m in range(3, 10)) < 2.0 ** -9 * p and c[3] * 0.5 ** 3 < 2.0 ** -9 * p
+    assert c[8] * 0.5 ** 8 < 2.0 ** -29 * p
