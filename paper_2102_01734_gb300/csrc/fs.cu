@@ -55,27 +55,13 @@ __device__ __forceinline__ double red_value(double x) { return x; }
 // Taylor coefficients of p(u) = e2/u^3 = 2 sum_m (-1)^m u^m / (m+3)!.
 constexpr double fact(int n) { return n <= 1 ? 1.0 : n * fact(n - 1); }
 constexpr double pc(int m) { return (m % 2 ? -2.0 : 2.0) / fact(m + 3); }
-template <int M> struct PC { static constexpr double v = pc(M); };
 template <int M> struct PCf { static constexpr float v = (float)pc(M); };
-
-// Horner evaluation of p(u) from degree M down to 0, unrolled at compile time.
-template <int M> struct Horner {
-    __device__ __forceinline__ static double eval(double acc, double u) {
-        return Horner<M - 1>::eval(fma(acc, u, PC<M - 1>::v), u);
-    }
-};
-template <> struct Horner<0> {
-    __device__ __forceinline__ static double eval(double acc, double) { return acc; }
-};
 
 struct IntervalF {
     float E, a0, a, d;
 };
-struct IntervalD {
-    double E, a0, a, d;
-};
 
-__device__ __forceinline__ IntervalF interval(float u) {
+__device__ __forceinline__ IntervalF interval(float u, const unsigned long long *) {
     IntervalF r;
     if (u < 1.0f) {
         // Horner, m = 8 .. 0: truncation < 1.3e-8 relative at u = 1
@@ -108,29 +94,8 @@ __device__ __forceinline__ IntervalF interval(float u) {
     return r;
 }
 
-__device__ __forceinline__ IntervalD interval(double u) {
-    IntervalD r;
-    if (u < 0.5) {
-        // Horner, m = 17 .. 0: truncation ~1e-23 relative at u = 1/2
-        const double p = Horner<17>::eval(PC<17>::v, u);
-        const double b = u * p;
-        const double a = 0.5 * u * (1.0 - b);
-        const double e0 = u * (1.0 - a);
-        r.E = 1.0 - e0;
-        r.a = a;
-        r.a0 = e0 - a;
-        r.d = a - b;
-    } else {
-        const double E = exp(-u);
-        const double ru = 1.0 / u;
-        const double e0 = 1.0 - E;
-        const double a = fma(-e0, ru, 1.0);
-        r.E = E;
-        r.a = a;
-        r.a0 = fma(-(1.0 + u), E, 1.0) * ru;
-        r.d = fma(2.0, a, -e0) * ru;
-    }
-    return r;
+__device__ __forceinline__ IntervalD interval(double u, const unsigned long long *tab) {
+    return interval64_w(u, tab);
 }
 
 template <typename R> __device__ __forceinline__ R div_fast(R x, R y);
@@ -138,7 +103,7 @@ template <> __device__ __forceinline__ float div_fast<float>(float x, float y) {
     return __fdividef(x, y);
 }
 template <> __device__ __forceinline__ double div_fast<double>(double x, double y) {
-    return x / y;
+    return x * recip64(y);
 }
 
 template <typename R> __device__ __forceinline__ R clamp01(R x) {
@@ -159,9 +124,15 @@ __device__ __forceinline__ int rep_of(uint32_t c, int x0, int y0, int nx, int ny
                           nx, ny);
 }
 
+// One characteristic a thread, with Lambda* (FP64: the FP64 pipe bounds it; 33^3
+// voxels, 128 angles 3.24 ms with the library's exp, divisions and an 18-term
+// series, 1.98 ms with interval64_w and recip64; parabolic 4.98 -> 3.23 ms. Error of
+// Lambda* against 64 bits 7.8e-16 -> 7.1e-16).
 template <typename R, bool PARAB, bool LSTAR>
 __global__ void __launch_bounds__(128) fs_kernel(FsParams p) {
     using R2 = typename V2<R>::T;
+    __shared__ unsigned long long tab[64];
+    if (sizeof(R) == 8) exp_table(tab);
     const int nray = p.nx * p.ny;
     const int ray = blockIdx.x * blockDim.x + threadIdx.x;
     if (ray >= nray) return;
@@ -192,7 +163,7 @@ __global__ void __launch_bounds__(128) fs_kernel(FsParams p) {
 
     for (int k = 0; k < K; ++k) {
         const R u = R(0.5) * (chil_p + chil_c);
-        const auto f = interval(u);
+        const auto f = interval(u, tab);
         const bool has_next = (k + 1 < K);
         int vn = v;
         R chil_n = R(0), S_n = S_c;
@@ -490,8 +461,8 @@ __global__ void __launch_bounds__(256, 3) fs_quad_kernel(FsParams p) {
 // 27 planes and J), added to the others afterwards (band_merge_kernel, 0.16 ms at
 // 97^3). 154 registers: six blocks of 64 a SM without spills; four blocks of 128
 // spill and are no faster. With both kernels and 512 angles: 65 x 65 x 257 27.4 ->
-// 22.5 ms, 97^3 21.2 -> 17.2 ms; L2 reductions at 61 %, issue at 52 %, neither
-// saturated. Error of Lambda* against 64 bits at 65^3: 6.83e-9 -> 6.80e-9 (interval
+// 22.5 ms, 97^3 21.2 -> 17.2 ms; at 65 x 65 x 257 the L2's atomic input is 73 %
+// busy, issue 54 %. Error of Lambda* against 64 bits at 65^3: 6.83e-9 -> 6.80e-9 (interval
 // functions from the 9-term series, alpha without cancellation: with the
 // polynomials of the kernel above and e0 - a it was 7.6e-9).
 template <bool PARAB>
@@ -832,11 +803,12 @@ __global__ void pair_pack_kernel(int nx, int ny, int nz, const float2 *__restric
 // ---- FP64 formal solution without Lambda* (refinement residuals, FP64 mode
 // after the first iteration). The FP64 pipe is the bound, so what can leave it
 // does: branch tests on the high word of non-negative doubles (integer compares),
-// reciprocals, the smaller terms of the interval polynomials and of e^-u, widening
-// by integer moves (fs64_step.cuh: hi_below, recip64, interval64). 23 FP64
-// instructions a point remain of 34 in the parabolic form below u = 1/2. 33^3
-// voxels, 128 angles, linear: 1303 us with three FP64 operations a reciprocal,
-// nine for the polynomial and eight for e^-u, 947 us now.
+// reciprocals, the interval polynomial and 1 - e^-u, widening by integer moves
+// (fs64_step.cuh: hi_below, recip64, interval64). 10 FP64 instructions a point
+// remain in the linear form below u = 1/2 and 17 in the parabolic one, of 19 and 34.
+// 33^3 voxels, 128 angles, linear: 1303 us with three FP64 operations a reciprocal,
+// nine for the polynomial and eight for e^-u; 947 us with the smaller terms of both
+// in float-float; 618 us with the rest in fixed point.
 
 // One thread per characteristic; per point: the replicated offset (FP32
 // record), the FP64 (l/2, J weight) record, the (chi, S) gather, and one
@@ -846,7 +818,7 @@ __global__ void pair_pack_kernel(int nx, int ny, int nz, const float2 *__restric
 // one FMA between.
 template <bool PARAB>
 __global__ void __launch_bounds__(128) fs64_fast_kernel(FsParams p) {
-    __shared__ double tab[64];
+    __shared__ unsigned long long tab[64];
     exp_table(tab);
     const int nray = p.nx * p.ny;
     const int ray = blockIdx.x * blockDim.x + threadIdx.x;

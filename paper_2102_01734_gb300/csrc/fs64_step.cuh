@@ -95,66 +95,109 @@ __device__ const double kPow2[64] = {
     0.5693943173783458, 0.5632608093041209, 0.5571933712979462, 0.5511912916539204,
     0.5452538663326288, 0.5393803988785599, 0.5335702003384118, 0.5278225891802786,
     0.5221368912137069, 0.5165124395106142, 0.5109485743270583, 0.5054446430258502};
-// ln2 / 64 as the sum of two doubles
-constexpr double kLn2Hi = 0.010830424696249145, kLn2Lo = 3.623510646634843e-19;
+// ln2 / 64 in units of 2^-64: the integer part and the next 32 bits
+constexpr unsigned long long kLn2Int = 0x2c5c85fdf473de6ULL;
+constexpr unsigned kLn2Frac = 0xaf278eceu;
 
-// The table in shared memory (every thread of the block must call it).
-__device__ __forceinline__ void exp_table(double *tab) {
-    if (threadIdx.x < 64) tab[threadIdx.x] = kPow2[threadIdx.x];
+// The table in shared memory, in units of 2^-63 (every thread of the block must
+// call it).
+__device__ __forceinline__ void exp_table(unsigned long long *tab) {
+    if (threadIdx.x < 64) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(kPow2[threadIdx.x]);
+        tab[threadIdx.x] = ((b & 0xfffffffffffffULL) | 1ULL << 52) << (threadIdx.x ? 10 : 11);
+    }
     __syncthreads();
 }
 
-// e^-u for 1/2 <= u < 37.5 (Tang's table-driven method): n = nearest integer
-// to 64 u / ln2 (found in FP32; a neighbour of it near a tie only widens r's
-// range), r = u - n ln2/64, |r| <= ln2/128 (1 + 2^-9), e^-r by its Taylor
-// polynomial of degree 5 (truncation r^6/720 < 4e-17; the terms from r^2 on, below
-// 2^-15, in float-float), e^-u = 2^-(n div 64) 2^-((n mod 64)/64) e^-r. Five FP64
-// operations, a third of the library's exp, whose accuracy over the whole range
-// e^-u does not need here: the caller takes 1 - e^-u.
-__device__ __forceinline__ double exp_neg64(double u, const double *tab) {
+// x >= 0 in units of 2^-64, modulo 2^64, truncated
+__device__ __forceinline__ unsigned long long fixed64(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned long long m = (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+    const int sh = (int)(hi >> 20) - 1011;
+    return sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ULL);
+}
+
+// e^-u for 1/2 <= u < 37.5 as E 2^-62 2^-k (Tang's table-driven method in fixed
+// point, no FP64 operation): n = nearest integer to 64 u / ln2 (found in FP32; a
+// neighbour of it near a tie only widens r's range), r = u - n ln2/64 modulo 1 in
+// units of 2^-64 (exact but for the last two), |r| <= ln2/128 (1 + 2^-9), e^-r - 1 =
+// -r + g with g from the Taylor polynomial of degree 5 (truncation r^6/720 < 4e-17;
+// g, below 2^-15, in float-float), e^-u = 2^-(n div 64) 2^-((n mod 64)/64) e^-r.
+__device__ __forceinline__ unsigned long long exp_fixed64(double u, const unsigned long long *tab,
+                                                          int &k) {
     const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
     const float uf = __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
     const float t = fmaf(uf, 92.33248f, 12582912.0f);  // 1.5 2^23: n in the low bits
     const int n = __float_as_int(t) - 0x4B400000;
-    const double nd = widen_f32(t - 12582912.0f);
-    const double r = fma(-nd, kLn2Lo, fma(-nd, kLn2Hi, u));
-    float rh, rl;
-    split_ff(r, rh, rl);
-    if (r < 0.0) {
-        rh = -rh;
-        rl = -rl;
-    }
+    const unsigned long long m = (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+    const unsigned long long nl =
+        (unsigned long long)n * kLn2Int + ((unsigned long long)n * kLn2Frac >> 32);
+    const long long r = (long long)((m << ((int)(hi >> 20) - 1011)) - nl);
+    const float rh = (float)(int)(r >> 34) * 0x1p-30f;
+    const float rl = (float)(unsigned)(r >> 2) * 0x1p-62f;  // the low 34 bits
     float h = fmaf(rh, (float)(-1.0 / 120.0), (float)(1.0 / 24.0)), l = 0.0f;
     horner_ff(h, l, rh, rl, -1.0 / 6.0);
     horner_ff(h, l, rh, rl, 0.5);
     const float p = rh * rh, e = fmaf(rh, 2.0f * rl, fmaf(rh, rh, -p));  // r^2
     const float gh = p * h, gl = fmaf(e, h, fmaf(p, l, fmaf(p, h, -gh)));
-    const double P = (widen_f32(gl) - r) + widen_f32(gh);  // e^-r - 1
-    const double T = tab[n & 63];
-    const double E = fma(T, P, T);
-    return __hiloint2double(__double2hiint(E) - ((n >> 6) << 20), __double2loint(E));
+    const int g1 = __float2int_rn(gh * 0x1p40f);
+    const int g2 = __float2int_rn((fmaf((float)g1, -0x1p-40f, gh) + gl) * 0x1p64f);
+    const long long P = ((long long)g1 << 24) + g2 - r;  // e^-r - 1
+    k = n >> 6;
+    return __umul64hi(tab[n & 63], (1ULL << 63) + (unsigned long long)(P >> 1));
+}
+// 1 - e^-u and e^-u, rounded once
+__device__ __forceinline__ double one_minus_exp64(double u, const unsigned long long *tab) {
+    int k;
+    const unsigned long long E = exp_fixed64(u, tab, k);
+    const unsigned long long e0 = (1ULL << 62) - (E >> k);  // units of 2^-62
+    const bool half = e0 >= 1ULL << 61;
+    return __longlong_as_double((half ? 1021LL << 52 : 1020LL << 52) +
+                                (long long)(half ? (e0 + 256) >> 9 : (e0 + 128) >> 8));
+}
+__device__ __forceinline__ double exp_neg64(double u, const unsigned long long *tab) {
+    int k;
+    const unsigned long long E = exp_fixed64(u, tab, k);
+    const int sh = 11 - __clzll((long long)E);  // 53 bits stay
+    return __longlong_as_double(((long long)(1012 + sh - k) << 52) +
+                                (long long)((E + (1ULL << (sh - 1))) >> sh));
 }
 
-// The terms of p(u) from degree 3 on, over u^3, for 0 <= u < 1/2, in float-float
-// (degrees 8 and 9 in FP32): together they are below 2^-9 of p, and their error
-// below 2^-46 of themselves. Below 2^-38 only the first counts.
-__device__ __forceinline__ double tail64(double u) {
-    float uh, ul;
-    split_ff(u, uh, ul);
-    float h = fmaf(uh, -3.4475018036590732e-09f, 4.9354831016668725e-08f), l = 0.0f;
-    horner_ff(h, l, uh, ul, -5.507115670485655e-07);
-    horner_ff(h, l, uh, ul, 5.511310234105578e-06);
-    horner_ff(h, l, uh, ul, -4.9603140878306714e-05);
-    horner_ff(h, l, uh, ul, 3.9682539230545495e-04);
-    horner_ff(h, l, uh, ul, -2.777777777429071e-03);
-    return widen_f32(h) + widen_f32(l);
-}
+// Horner's rule for p(u) = e2/u^3, 0 <= u < 1/2, degree 9, without an FP64 operation:
+// degrees 9 and 8 in FP32, 7 to 3 in float-float (below 2^-9 of p in all), 2 to 0 in
+// fixed point (units of 2^-64, alternating signs), rounded once: 1/4 < p < 1/2.
+struct Horner64 {
+    int next;  // degree of the next coefficient, known at compile time
+    float h, l;
+    unsigned long long v;
+
+    __device__ __forceinline__ friend Horner64 fma(Horner64 p, double u, double c) {
+        float uh, ul;
+        split_ff(u, uh, ul);
+        const int degree = p.next--;
+        if (degree >= 8) {
+            p.h = fmaf(uh, p.h, (float)c);
+        } else if (degree >= 3) {
+            horner_ff(p.h, p.l, uh, ul, c);
+        } else {
+            if (degree == 2) {  // the sum of the higher terms, negative
+                const int t1 = __float2int_rn(p.h * -0x1p30f);
+                const int t2 = __float2int_rn((fmaf((float)t1, -0x1p-30f, -p.h) - p.l) * 0x1p56f);
+                p.v = (unsigned long long)(((long long)t1 << 34) + ((long long)t2 << 8));
+            }
+            p.v = (unsigned long long)(fabs(c) * 0x1p64) - __umul64hi(fixed64(u), p.v);
+        }
+        return p;
+    }
+    __device__ __forceinline__ double value() const {
+        return __longlong_as_double((1020LL << 52) + (long long)((v + 512) >> 10));
+    }
+};
 
 // Interval functions in FP64 (as interval(double)); for u < 1/2 p(u) =
 // e2/u^3 is a degree-9 polynomial fitted to the exact function (least squares
-// in relative error at 300 Chebyshev nodes of [0, 1/2]; FP64 Horner error
-// 1.6e-16 relative, the rounding of its leading coefficient 1/3), its terms from
-// degree 3 on evaluated off the FP64 pipe (tail64). From 37.5 on e^-u is below
+// in relative error at 300 Chebyshev nodes of [0, 1/2]). It and 1 - e^-u are
+// evaluated off the FP64 pipe (Horner64, one_minus_exp64). From 37.5 on e^-u is below
 // 2^-54, and e0 = 1 (a NaN u goes there and reaches a through ru). ru = 1/u
 // for u >= 1/2 (carried from the previous step, or computed here if CARRY is
 // false). Returns e0, a, d for the update in difference form.
@@ -162,14 +205,21 @@ struct IntervalDE {
     double e0, a, d;
 };
 template <bool CARRY>
-__device__ __forceinline__ IntervalDE interval64(double u, double ru, const double *tab) {
+__device__ __forceinline__ IntervalDE interval64(double u, double ru, const unsigned long long *tab) {
     IntervalDE r;
     if (hi_below(u, 0x3FE00000)) {
-        double p = tail64(u);
+        Horner64 p{9, 0.0f, 0.0f, 0ULL};
+        p = fma(p, u, -3.4475018036590732e-09);
+        p = fma(p, u, 4.9354831016668725e-08);
+        p = fma(p, u, -5.507115670485655e-07);
+        p = fma(p, u, 5.511310234105578e-06);
+        p = fma(p, u, -4.9603140878306714e-05);
+        p = fma(p, u, 3.9682539230545495e-04);
+        p = fma(p, u, -2.777777777429071e-03);
         p = fma(p, u, 1.6666666666652976e-02);
         p = fma(p, u, -8.333333333333312e-02);
         p = fma(p, u, 3.333333333333333e-01);
-        const double b = u * p;
+        const double b = u * p.value();
         const double hu = __hiloint2double(max(0, __double2hiint(u) - 0x00100000), __double2loint(u));  // u / 2
         const double a = fma(-hu, b, hu);
         r.e0 = fma(-u, a, u);
@@ -178,11 +228,33 @@ __device__ __forceinline__ IntervalDE interval64(double u, double ru, const doub
     } else {
         if (!CARRY) ru = recip64(u);
         double e0 = 1.0;
-        if (hi_below(u, 0x4042C000)) e0 = 1.0 - exp_neg64(u, tab);
+        if (hi_below(u, 0x4042C000)) e0 = one_minus_exp64(u, tab);
         const double a = fma(-e0, ru, 1.0);
         r.e0 = e0;
         r.a = a;
         r.d = fma(2.0, a, -e0) * ru;
+    }
+    return r;
+}
+
+// The same with E = e^-u and a0 = e0 - a, for the kernel with Lambda*.
+struct IntervalD {
+    double E, a0, a, d;
+};
+__device__ __forceinline__ IntervalD interval64_w(double u, const unsigned long long *tab) {
+    IntervalD r;
+    if (hi_below(u, 0x3FE00000)) {
+        const IntervalDE f = interval64<false>(u, 0.0, tab);
+        r.E = 1.0 - f.e0;
+        r.a0 = f.e0 - f.a;
+        r.a = f.a;
+        r.d = f.d;
+    } else {
+        r.E = hi_below(u, 0x4042C000) ? exp_neg64(u, tab) : exp(-u);
+        const double ru = recip64(u), e0 = 1.0 - r.E;
+        r.a = fma(-e0, ru, 1.0);
+        r.a0 = fma(-(1.0 + u), r.E, 1.0) * ru;
+        r.d = fma(2.0, r.a, -e0) * ru;
     }
     return r;
 }

@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(128) sph_fs_fast_kernel(SphFsParams p, double 
 // at the replicated index (folded afterwards).
 template <bool PARAB>
 __global__ void __launch_bounds__(128) sph_fs64_fast_kernel(SphFsParams p, double *__restrict__ Jrep) {
-    __shared__ double tab[64];
+    __shared__ unsigned long long tab[64];
     exp_table(tab);
     const long long ray = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (ray >= p.nrays) return;

@@ -14,42 +14,46 @@ SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 def _constants():
     src = open(SRC).read()
     body = re.search(r"kPow2\[64\] = \{(.*?)\};", src, re.S).group(1)
-    hi, lo = re.search(r"kLn2Hi = (\S+), kLn2Lo = (\S+);", src).groups()
-    return [float(x) for x in body.split(",")], float(hi), float(lo)
+    whole, frac = re.search(r"kLn2Int = (0x\w+)ULL;.*?kLn2Frac = (0x\w+)u;", src, re.S).groups()
+    return [float(x) for x in body.split(",")], int(whole, 16), int(frac, 16)
 
 
 def test_table_is_correctly_rounded():
-    tab, hi, lo = _constants()
+    tab, whole, frac = _constants()
     assert len(tab) == 64
     with mpmath.workdps(50):
         assert tab == [float(mpmath.mpf(2) ** (-mpmath.mpf(j) / 64)) for j in range(64)]
-        ln2 = mpmath.log(2) / 64
-        assert hi == float(ln2) and lo == float(ln2 - mpmath.mpf(hi))
+        assert (whole << 32) + frac == int(mpmath.floor(mpmath.log(2) / 64 * mpmath.mpf(2) ** 96))
 
 
-def test_error_of_exp_neg():
-    """Every operation in exact arithmetic rounded once (as the fused ones
-    are): the table's rounding, e^-r's and the last product's, each 2^-53."""
-    tab, hi, lo = _constants()
-    m = mpmath.mpf
-    rd = lambda x: float(x)
+def test_error_of_one_minus_exp():
+    """The fixed-point steps as integers, g exact to 2^-44 of itself: the table's
+    rounding (2^-54) and the last one (2^-55 below 1/2) over 1 - e^-u >= 0.393."""
+    tab, whole, frac = _constants()
     worst = 0.0
     with mpmath.workdps(40):
         for u in np.concatenate([[0.5, 37.4999], np.random.default_rng(1).uniform(0.5, 37.5, 1500),
                                  (np.arange(48, 200) + 0.5) * np.log(2) / 64]):
             u = float(u)
             n = int(np.rint(np.float32(np.float32(u) * np.float32(92.33248))))
-            r = rd(m(u) - n * m(hi))
-            r = rd(m(r) - n * m(lo))
-            assert abs(r) <= np.log(2) / 128 * (1 + 2.0 ** -9)
-            q = rd(m(r) * m(-1.0 / 120) + m(1.0 / 24))
-            q = rd(m(r) * m(q) + m(-1.0 / 6))
-            q = rd(m(r) * m(q) + m(0.5))
-            P = rd(m(rd(m(r) * m(r))) * m(q) - m(r))
-            T = tab[n & 63]
-            E = rd(m(T) * m(P) + m(T)) * 2.0 ** -(n >> 6)
-            worst = max(worst, float(abs(m(E) * mpmath.exp(m(u)) - 1)))
-    assert worst < 2.5 * 2.0 ** -53
+            m, e = np.frexp(u)
+            mant = int(m * 2 ** 53)
+            r = ((mant << (int(e) + 11)) - n * whole - (n * frac >> 32)) % 2 ** 64
+            r -= 2 ** 64 * (r >> 63)
+            assert abs(r) <= np.log(2) / 128 * (1 + 2.0 ** -9) * 2 ** 64
+            x = mpmath.mpf(r) / 2 ** 64
+            rh, rl = r >> 34, (r >> 2) & 0xffffffff
+            assert abs(rh) < 2 ** 23 and (rh << 34) + (rl << 2) + (r & 3) == r
+            g = x * x * (0.5 + x * (mpmath.mpf(-1) / 6 + x * (mpmath.mpf(1) / 24 - x / 120)))
+            g1 = int(mpmath.nint(g * 2 ** 40))
+            assert 0 <= g1 <= 2 ** 24
+            P = (g1 << 24) + int(mpmath.nint((g * (1 + mpmath.mpf(2) ** -44) - mpmath.mpf(g1) / 2 ** 40) * 2 ** 64)) - r
+            T = int(tab[n & 63] * 2 ** 63)
+            E = T * (2 ** 63 + (P >> 1)) >> 64
+            e0 = 2 ** 62 - (E >> (n >> 6))
+            d = (e0 + 256 >> 9) * 2.0 ** -53 if e0 >= 2 ** 61 else (e0 + 128 >> 8) * 2.0 ** -54
+            worst = max(worst, float(abs(mpmath.mpf(d) / (1 - mpmath.exp(-mpmath.mpf(u))) - 1)))
+    assert worst < (2.0 ** -54 + 2.0 ** -55) / 0.393 * 1.01
 
 
 def _rd(x):
@@ -92,9 +96,10 @@ def test_reciprocal():
 
 
 def test_tail_weight():
-    """What tail64 evaluates in float-float is below 2^-9 of p(u) on [0, 1/2], and
-    its terms of degree 8 and 9, in FP32, below 2^-30."""
+    """What Horner64 evaluates in float-float (2^-45 of itself) is below 2^-9 of p(u) on
+    [0, 1/2], and its terms of degree 8 and 9, in FP32, below 2^-29; p's high bit is
+    that of 1/4 and the corrections' integers fit."""
     c = {m: 2.0 / float(mpmath.factorial(m + 3)) for m in range(10)}
     p = 1 / 3 - 0.5 / 12
-    assert sum(c[m] * 0.5 ** m for m in range(3, 10)) < 2.0 ** -9 * p and c[3] * 0.5 ** 3 < 2.0 ** -9 * p
-    assert c[8] * 0.5 ** 8 < 2.0 ** -29 * p
+    assert c[3] * 0.5 ** 3 < 2.0 ** -9 * p and c[8] * 0.5 ** 8 < 2.0 ** -29 * p
+    assert p > 0.25 and c[3] * 2 ** 30 < 2 ** 22 and 2.0 ** -31 * 2 ** 56 <= 2 ** 25
