@@ -72,8 +72,8 @@ FS_KERNEL = {1: "fs_fast_kernel", 2: "fs_pair_kernel", 4: "fs_quad_kernel"}
 FS_SOURCES = ("paper_2102_01734_gb300/csrc/fs.cu", "paper_2102_01734_gb300/csrc/fs_step.cuh",
               "paper_2102_01734_gb300/csrc/fs64_step.cuh",
               "paper_2102_01734_gb300/csrc/rt3d_internal.cuh")
-FS_PROFILE = "profiles/fs_pair_kernel_box129_field.md"
-FS_PROFILE_KERNEL = "fs_pair_kernel"
+FS_PROFILE = "profiles/fs_quad_kernel_box129_field.md"
+FS_PROFILE_KERNEL = "fs_quad_kernel"
 
 
 def fs_source_hash() -> str:

@@ -47,7 +47,8 @@ typedef enum {
     RT3D_ECUDA = 3,          /* a CUDA call failed */
     RT3D_ENOTCONVERGED = 4,  /* iteration cap reached; J holds the last iterate */
     RT3D_ETIMEOUT = 5,       /* reserved for a bounded device-side wait that ran out;
-                                no kernel of this library spins on the device */
+                                the kernels wait at the barriers of cooperative launches
+                                and of clusters only, whose blocks are all resident */
     RT3D_ENUMERIC = 6        /* NaN/Inf met in a residual or change */
 } rt3d_status;
 

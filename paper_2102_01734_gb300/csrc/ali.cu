@@ -9,9 +9,11 @@
 // their 26 planes contiguous, os_coef_index) and stores 1/diag in FP64.
 // A sweep reads the coefficients once (the HBM stream that bounds it), the
 // neighbours of dJ through L1/L2, and writes dJ^{m+1} with the two maxima
-// of the stop test. Sweeps are launched back to back; each reads the
-// previous sweep's maxima and returns at once after the stop test is met,
-// so a fixed launch sequence serves any sweep count.
+// of the stop test. A grid whose coefficients fit in the chip's shared memory is
+// solved in one cooperative launch (os_resident_kernel); elsewhere sweeps are
+// launched back to back (Gauss-Seidel: two launches a sweep), each reads the
+// previous sweep's maxima and returns at once after the stop test is met, so a
+// fixed launch sequence serves any sweep count.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -252,7 +254,8 @@ __global__ void __launch_bounds__(256) gs_colour_kernel(int nx, int ny, int nz, 
 // Sweep at 129^3 149 us with one launch per colour (gs_colour_kernel), 100 us
 // here; at 65^3 56 and 35 us. What bounds it is the latency of a voxel's
 // instructions at 16 warps per SM: a ring of coefficient blocks in shared memory
-// (cp.async) ran at 14 warps and 118 us, two smaller blocks per SM at 110 us.
+// (cp.async) ran at 14 warps and 118 us, two smaller blocks per SM at 110 us,
+// prefetches of the next colour's coefficients into the L2 at 117 us.
 template <typename A> struct GsShared {
     int pitch, rows;  // row pitch (nx + 2), rows of a plane (2 band + 2)
     __host__ __device__ int plane() const { return rows * pitch; }
