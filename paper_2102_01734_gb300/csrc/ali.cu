@@ -1136,18 +1136,26 @@ cudaError_t launch_os_resident(int nx, int ny, int nz, bool gs, const void *a, b
     *ran = nx < 2048 && ny < 2048 && nz < 512 &&
            (a64 ? os_resident_shape<double>(N, gs, cg, &grid) : os_resident_shape<float>(N, gs, cg, &grid));
     if (!*ran) return cudaSuccess;
+    cudaError_t e;
     if (a64) {
         const double *x = static_cast<const double *>(a);
-        return gs ? os_resident<double, true>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf[0], buf[1],
-                                              max_sweeps, tol, st, s, per)
-                  : os_resident<double, false>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf[0], buf[1],
-                                               max_sweeps, tol, st, s, per);
+        e = gs ? os_resident<double, true>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf[0], buf[1],
+                                           max_sweeps, tol, st, s, per)
+               : os_resident<double, false>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf[0], buf[1],
+                                            max_sweeps, tol, st, s, per);
+    } else {
+        const float *x = static_cast<const float *>(a);
+        e = gs ? os_resident<float, true>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf32[0], buf32[1],
+                                          max_sweeps, tol, st, s, per)
+               : os_resident<float, false>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf32[0], buf32[1],
+                                           max_sweeps, tol, st, s, per);
     }
-    const float *x = static_cast<const float *>(a);
-    return gs ? os_resident<float, true>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf32[0], buf32[1],
-                                         max_sweeps, tol, st, s, per)
-              : os_resident<float, false>(nx, ny, nz, cg, grid, x, inv_diag, r, buf, buf32[0], buf32[1],
-                                          max_sweeps, tol, st, s, per);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the SMs is not ours: sweep by sweep
+        cudaGetLastError();
+        *ran = false;
+        return cudaSuccess;
+    }
+    return e;
 }
 
 cudaError_t launch_bicg_init(int n, const double *r, const BicgVecs &v, BicgState *bs,
