@@ -20,6 +20,12 @@
 // 113 -> 42 us), the 11 weight gradients 1820 -> 277 us and the bias gradients,
 // 168 us in launches of their own, inside them. A whole training step 3.76 ->
 // 0.92 ms.
+//
+// The sums run over blocks of 16 channels, the 27 taps inside. Against gradients
+// in 64 bits, over 25 training steps on boxes of different sizes and 22 tensors
+// each, the mean error is that of the taps-first order (ratio 0.999, per-tensor
+// medians 0.97 to 1.02); a tensor of one step scatters either way, up to a factor of
+// a few where its error is small, because BF16 roundings of the activations flip.
 #include "nn_conv.cuh"
 
 #include <algorithm>
