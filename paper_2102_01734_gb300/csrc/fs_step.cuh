@@ -262,6 +262,11 @@ __device__ __forceinline__ IntervalN2 interval_both(float2 u) {
 __device__ __forceinline__ float2 linear_n(const RayN &s, const IntervalN2 &f) {
     return fma2(f.na, s.nD, fma2(f.e0, sub2(s.Sp, s.I), s.I));
 }
+// The blend weight f given -q
+__device__ __forceinline__ float2 blend_n(float2 u, float2 nq) {
+    return mul2(pk(__saturatef(fmaf(-2.0f, u.x, 2.0f)), __saturatef(fmaf(-2.0f, u.y, 2.0f))),
+                pk(__saturatef(fmaf(0.5f, nq.x, 2.0f)), __saturatef(fmaf(0.5f, nq.y, 2.0f))));
+}
 // f s d (dS - q dSn), both factors negated, added to In; w the next interval.
 // The two divisions share one reciprocal: with X = wf (u + wf), u/wf = u (u +
 // wf)/X and u/(u + wf) = u wf/X, wf = w floored at 1e-15 (X stays a normal FP32
@@ -273,9 +278,21 @@ __device__ __forceinline__ float2 parabola_n(const RayN &s, const IntervalN2 &f,
     const float2 X = mul2(nwf, nuw);
     const float2 uR = mul2(s.u, pk(rcp_approx(X.x), rcp_approx(X.y)));
     const float2 nq = mul2(nuw, uR), ns = mul2(nwf, uR);  // -u/wf, -u/(u + wf)
-    const float2 fw = mul2(pk(__saturatef(fmaf(-2.0f, s.u.x, 2.0f)), __saturatef(fmaf(-2.0f, s.u.y, 2.0f))),
-                           pk(__saturatef(fmaf(0.5f, nq.x, 2.0f)), __saturatef(fmaf(0.5f, nq.y, 2.0f))));
-    return fma2(mul2(mul2(fw, f.d), ns), fma2(nq, nDn, s.nD), In);
+    return fma2(mul2(mul2(blend_n(s.u, nq), f.d), ns), fma2(nq, nDn, s.nD), In);
+}
+// The same ratios, -u/w and -u/(u + w), over the whole range of optical depths: a
+// reciprocal each, w floored near the smallest normal number only. Bounded by 4
+// (from there on the blend weight is 0) and 1, they are finite for infinite u and w
+// and for w = 0 too, so that a zero blend weight leaves nothing. (From one
+// reciprocal of w (u + w), as above, the floor has to be 1e-15, below which the
+// parabola of a transparent cell is lost: there up to 0.3 % of its emission.)
+__device__ __forceinline__ void ratios_n(float2 u, float2 w, float2 &nq, float2 &ns) {
+    const float2 nw = pk(fminf(-w.x, -1e-37f), fminf(-w.y, -1e-37f));
+    const float2 nuw = sub2(nw, u);
+    const float2 q = mul2(u, pk(rcp_approx(nw.x), rcp_approx(nw.y)));
+    const float2 s = mul2(u, pk(rcp_approx(nuw.x), rcp_approx(nuw.y)));
+    nq = pk(fmaxf(q.x, -4.0f), fmaxf(q.y, -4.0f));
+    ns = pk(fmaxf(s.x, -1.0f), fmaxf(s.y, -1.0f));
 }
 // One point of two pairs (all lanes of the warp): s[j].I becomes the
 // intensities at the current point, the rest moves to the next point (c[j] its
@@ -417,16 +434,10 @@ __device__ __forceinline__ bool quad_advance_w(RayN (&s)[2], const float4 (&c)[2
             if (!all_thin) f = select_w(u, f, wt[j]);
             float2 In = linear_n(s[j], f);
             float2 g = pk1(0.0f), qg = pk1(0.0f);  // -f s d and q f s d
-            if (PARAB) {  // as parabola_n
-                const float2 nwf = pk(fminf(-w[j].x, -1e-15f), fminf(-w[j].y, -1e-15f));
-                const float2 nuw = sub2(nwf, u);
-                const float2 nq = mul2(u, pk(rcp_approx(nwf.x), rcp_approx(nwf.y)));
-                const float2 ns = mul2(u, pk(rcp_approx(nuw.x), rcp_approx(nuw.y)));
-                const float2 fw = mul2(pk(__saturatef(fmaf(-2.0f, u.x, 2.0f)),
-                                          __saturatef(fmaf(-2.0f, u.y, 2.0f))),
-                                       pk(__saturatef(fmaf(0.5f, nq.x, 2.0f)),
-                                          __saturatef(fmaf(0.5f, nq.y, 2.0f))));
-                g = mul2(mul2(fw, f.d), ns);
+            if (PARAB) {
+                float2 nq, ns;
+                ratios_n(u, w[j], nq, ns);
+                g = mul2(mul2(blend_n(u, nq), f.d), ns);
                 qg = mul2(nq, g);
                 In = fma2(g, fma2(nq, nDn[j], s[j].nD), In);
             }
@@ -479,9 +490,6 @@ __device__ __forceinline__ void twin_start(RayT &s, float2 cs, float hl, float I
 template <bool PARAB>
 __device__ __forceinline__ void twin_coef(float2 u, float2 w, float2 nD, float2 nDn, float2 &e0,
                                           float2 &B) {
-    RayN r;
-    r.u = u;
-    r.nD = nD;
     IntervalN2 f;
     const bool tx = !(u.x < 1.0f), ty = !(u.y < 1.0f);
     if (tx && ty) {
@@ -493,7 +501,11 @@ __device__ __forceinline__ void twin_coef(float2 u, float2 w, float2 nD, float2 
     f = tx || ty ? interval_both(u) : interval_thin(u);
     e0 = f.e0;
     B = mul2(f.na, nD);
-    if (PARAB) B = parabola_n(r, f, w, nDn, B);
+    if (PARAB) {
+        float2 nq, ns;
+        ratios_n(u, w, nq, ns);
+        B = fma2(mul2(mul2(blend_n(u, nq), f.d), ns), fma2(nq, nDn, nD), B);
+    }
 }
 // Points k and k + 1, given (chi, S) of points k + 1 and k + 2 and their half
 // chords; moves on to k + 2 and returns the two intensities.
