@@ -5,7 +5,10 @@
 // compound operations follow the "sloppy" double-double algorithms of Hida,
 // Li and Bailey (2001): relative error a few units of 2^-48 except under
 // cancellation, where the error stays a few units of 2^-48 of the operands.
-// Every product that must stay unfused is written with fmaf explicitly.
+// What has to be rounded by itself is written with __fmul_rn, __fadd_rn and
+// __fsub_rn, which the compiler does not fuse (a plain product may be fused into
+// whatever sum it enters, here or in a caller, and the error terms then count its
+// low part twice).
 #pragma once
 
 namespace rt3d {
@@ -24,18 +27,18 @@ __device__ __forceinline__ ff ff_split(double x) {
 }
 
 __device__ __forceinline__ ff two_sum(float a, float b) {
-    const float s = a + b;
-    const float v = s - a;
-    return ff{s, (a - (s - v)) + (b - v)};
+    const float s = __fadd_rn(a, b);
+    const float v = __fsub_rn(s, a);
+    return ff{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v))};
 }
 
 __device__ __forceinline__ ff quick_two_sum(float a, float b) {
-    const float s = a + b;
-    return ff{s, b - (s - a)};
+    const float s = __fadd_rn(a, b);
+    return ff{s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
 __device__ __forceinline__ ff two_prod(float a, float b) {
-    const float p = a * b;
+    const float p = __fmul_rn(a, b);
     return ff{p, fmaf(a, b, -p)};
 }
 
@@ -110,7 +113,8 @@ __device__ __forceinline__ ff ff_recip(ff x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x.hi));
     const float e = fmaf(-x.lo, r, fmaf(-x.hi, r, 1.0f));
-    return quick_two_sum(r, r * fmaf(e, e, e));
+    const float g = fmaf(e, e, e), s = fmaf(r, g, r);
+    return ff{s, fmaf(r, g, __fsub_rn(r, s))};
 }
 
 // FP64 value of a float-float (the widening of each part is exact; the sum

@@ -19,10 +19,11 @@ __device__ __forceinline__ bool hi_below(double x, int b_hi) {
     return (unsigned)__double2hiint(x) < (unsigned)b_hi;
 }
 
-// a + b = s + t exactly (Knuth)
+// a + b = s + t exactly (Knuth). Here and below, what has to be rounded by itself is
+// written with __fmul_rn, __fadd_rn and __fsub_rn: the compiler fuses none of them.
 __device__ __forceinline__ float sum_exact(float a, float b, float &t) {
-    const float s = a + b, bb = s - a;
-    t = (a - (s - bb)) + (b - bb);
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    t = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
     return s;
 }
 
@@ -41,14 +42,14 @@ __device__ __forceinline__ double recip64(double x) {
     const float xh = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
     const float xl = (float)(lo & 0x1fffffe0u) * 0x1p-52f, xt = (float)(lo & 31u) * 0x1p-52f;
     const float r0 = rcp_approx(xh);
-    const float ph = xh * r0, pl = fmaf(xh, r0, -ph);
-    const float q = xl * r0, ql = fmaf(xl, r0, -q);
+    const float ph = __fmul_rn(xh, r0), pl = fmaf(xh, r0, -ph);
+    const float q = __fmul_rn(xl, r0), ql = fmaf(xl, r0, -q);
     float t1, t2;
-    const float s1 = sum_exact(1.0f - ph, -q, t1);
+    const float s1 = sum_exact(__fsub_rn(1.0f, ph), -q, t1);
     const float eh = sum_exact(s1, -pl, t2);
     const float el = fmaf(-xt, r0, (t1 + t2) - ql);
     const float f = fmaf(eh, eh, el);
-    const float ch = r0 * eh, cl = fmaf(r0, f, fmaf(r0, eh, -ch));
+    const float ch = __fmul_rn(r0, eh), cl = fmaf(r0, f, fmaf(r0, eh, -ch));
     // r0 2^60, the correction's first 23 bits and the rest
     const int c1 = __float2int_rn(ch * 0x1p44f);
     const int c2 = __float2int_rn((fmaf((float)c1, -0x1p-44f, ch) + cl) * 0x1p60f);
@@ -61,10 +62,10 @@ __device__ __forceinline__ double recip64(double x) {
 // (h, l) = c + u (h, l) in float-float, |c| > |u h|
 __device__ __forceinline__ void horner_ff(float &h, float &l, float uh, float ul, double c) {
     const float chi = (float)c, clo = (float)(c - (double)chi);  // folded at compile time
-    const float p = uh * h;
+    const float p = __fmul_rn(uh, h);
     const float e = fmaf(uh, l, fmaf(ul, h, fmaf(uh, h, -p)));
-    const float s = chi + p;
-    l = (p - (s - chi)) + (e + clo);
+    const float s = __fadd_rn(chi, p);
+    l = __fadd_rn(__fsub_rn(p, __fsub_rn(s, chi)), __fadd_rn(e, clo));
     h = s;
 }
 // |x| as a pair of FP32 values, x = +-(h + l) to 2^-48 of it, by integer moves;
@@ -138,8 +139,8 @@ __device__ __forceinline__ unsigned long long exp_fixed64(double u, const unsign
     float h = fmaf(rh, (float)(-1.0 / 120.0), (float)(1.0 / 24.0)), l = 0.0f;
     horner_ff(h, l, rh, rl, -1.0 / 6.0);
     horner_ff(h, l, rh, rl, 0.5);
-    const float p = rh * rh, e = fmaf(rh, 2.0f * rl, fmaf(rh, rh, -p));  // r^2
-    const float gh = p * h, gl = fmaf(e, h, fmaf(p, l, fmaf(p, h, -gh)));
+    const float p = __fmul_rn(rh, rh), e = fmaf(rh, 2.0f * rl, fmaf(rh, rh, -p));  // r^2
+    const float gh = __fmul_rn(p, h), gl = fmaf(e, h, fmaf(p, l, fmaf(p, h, -gh)));
     const int g1 = __float2int_rn(gh * 0x1p40f);
     const int g2 = __float2int_rn((fmaf((float)g1, -0x1p-40f, gh) + gl) * 0x1p64f);
     const long long P = ((long long)g1 << 24) + g2 - r;  // e^-r - 1
