@@ -195,6 +195,14 @@ struct Horner64 {
     }
 };
 
+// u / 2 for finite u >= 0, by integer moves: one less in the exponent, or (below
+// 2^-1021, truncated to the smallest subnormal) the whole pattern shifted.
+__device__ __forceinline__ double half64(double u) {
+    const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
+    const bool low = hi < 0x00200000u;
+    return __hiloint2double((int)(low ? hi >> 1 : hi - 0x00100000u), (int)(low ? lo >> 1 | hi << 31 : lo));
+}
+
 // Interval functions in FP64 (as interval(double)); for u < 1/2 p(u) =
 // e2/u^3 is a degree-9 polynomial fitted to the exact function (least squares
 // in relative error at 300 Chebyshev nodes of [0, 1/2]). It and 1 - e^-u are
@@ -221,7 +229,7 @@ __device__ __forceinline__ IntervalDE interval64(double u, double ru, const unsi
         p = fma(p, u, -8.333333333333312e-02);
         p = fma(p, u, 3.333333333333333e-01);
         const double b = u * p.value();
-        const double hu = __hiloint2double(max(0, __double2hiint(u) - 0x00100000), __double2loint(u));  // u / 2
+        const double hu = half64(u);
         const double a = fma(-hu, b, hu);
         r.e0 = fma(-u, a, u);
         r.a = a;

@@ -129,3 +129,13 @@ def test_intervals(run):
     assert _err(out[6][u < 700], [e for e, v in zip(E, u) if v < 700]) < 2.4
     zero = run(np.array([0.0]))[:, 0]
     assert np.all(zero[[3, 4, 5, 7, 8, 9]] == 0.0) and zero[6] == 1.0
+
+
+def test_smallest(run):
+    """Down to the subnormals e0 = u and a = u/2, to the last unit."""
+    u = np.concatenate([2.0 ** -np.arange(1015.0, 1075.0), np.random.default_rng(8).uniform(0, 1e-307, 500),
+                        [2.2250738585072014e-308, 2.225073858507201e-308, 4.45e-308]])
+    out = run(u)
+    assert np.array_equal(out[3], u)
+    for k in (4, 8):
+        assert np.all(np.abs(out[k] - 0.5 * u) <= 5e-324)
