@@ -17,6 +17,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "rt3d_internal.cuh"
 
@@ -1030,17 +1031,18 @@ static bool gs_plane_shape(int nx, int ny, int nz, Periodic per, int *ranks, int
     return false;
 }
 
+// The planes of both parities in turn; returns how many colours have been launched:
+// all eight, or fewer (0, 4) where a launch is refused.
 template <typename A, bool SEAM>
-static cudaError_t gs_planes(int nx, int ny, int nz, const ColourGeo &cg, int ranks, int band,
-                             const GsShared<A> &g, const A *a, const double *inv_diag, const double *r,
-                             const double *src, double *dst, const float *src32, float *dst32, int m,
-                             double tol, OsState *st, cudaStream_t s, Periodic per) {
+static int gs_planes(int nx, int ny, int nz, const ColourGeo &cg, int ranks, int band,
+                     const GsShared<A> &g, const A *a, const double *inv_diag, const double *r,
+                     const double *src, double *dst, const float *src32, float *dst32, int m, double tol,
+                     OsState *st, cudaStream_t s, Periodic per) {
     const size_t shm = g.bytes();
-    if (shm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            gs_plane_kernel<A, SEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        if (e != cudaSuccess) return e;
-    }
+    if (shm > 48 * 1024 &&
+        cudaFuncSetAttribute(gs_plane_kernel<A, SEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)shm) != cudaSuccess)
+        return 0;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = ranks;
@@ -1053,36 +1055,35 @@ static cudaError_t gs_planes(int nx, int ny, int nz, const ColourGeo &cg, int ra
     lc.numAttrs = 1;
     for (int pz = 0; pz < 2 && pz < nz; ++pz) {
         lc.gridDim = dim3((nz - pz + 1) / 2 * ranks);
-        const cudaError_t e =
-            cudaLaunchKernelEx(&lc, gs_plane_kernel<A, SEAM>, nx, ny, nz, cg, pz, band, g, a, inv_diag, r,
-                               src, dst, src32, dst32, m, tol, st, per);
-        if (e != cudaSuccess) return e;
+        if (cudaLaunchKernelEx(&lc, gs_plane_kernel<A, SEAM>, nx, ny, nz, cg, pz, band, g, a, inv_diag, r,
+                               src, dst, src32, dst32, m, tol, st, per) != cudaSuccess)
+            return 4 * pz;
     }
-    return cudaSuccess;
+    return 8;
 }
 
 cudaError_t launch_gs_sweep(int nx, int ny, int nz, const ColourGeo &cg, const void *a, bool a64,
                             const double *inv_diag, const double *r, const double *src,
                             double *dst, const float *src32, float *dst32, int m, double tol,
                             OsState *st, cudaStream_t s, Periodic per, int *launches) {
-    cudaError_t e = cudaSuccess;
-    auto planes = [&](auto coef, const auto *x) -> bool {
-        using A = decltype(coef);
+    auto planes = [&](const auto *x) -> int {
+        using A = std::remove_const_t<std::remove_pointer_t<decltype(x)>>;
         int ranks = 0, band = 0;
         GsShared<A> g{};
-        if (!gs_plane_shape<A>(nx, ny, nz, per, &ranks, &band, &g)) return false;
-        *launches = nz > 1 ? 2 : 1;
+        if (!gs_plane_shape<A>(nx, ny, nz, per, &ranks, &band, &g)) return 0;
         const bool seam = (per.x && (nx & 1)) || (per.y && (ny & 1));
-        e = seam ? gs_planes<A, true>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
-                                      dst32, m, tol, st, s, per)
-                 : gs_planes<A, false>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
-                                       dst32, m, tol, st, s, per);
-        return true;
+        return seam ? gs_planes<A, true>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
+                                         dst32, m, tol, st, s, per)
+                    : gs_planes<A, false>(nx, ny, nz, cg, ranks, band, g, x, inv_diag, r, src, dst, src32,
+                                          dst32, m, tol, st, s, per);
     };
-    if (a64 ? planes(0.0, static_cast<const double *>(a)) : planes(0.0f, static_cast<const float *>(a)))
-        return e;
-    *launches = 8;
-    for (int c = 0; c < 8; ++c) {
+    const int first = a64 ? planes(static_cast<const double *>(a)) : planes(static_cast<const float *>(a));
+    *launches = first == 8 && nz == 1 ? 1 : first / 4 + (8 - first);
+    if (first == 8) return cudaSuccess;
+    // colour by colour, also where a cluster is refused (part of the SMs is not
+    // ours); what ails more than the cluster shows in these launches too
+    cudaGetLastError();
+    for (int c = first; c < 8; ++c) {
         const int blocks = grid_for(cg.cnt[c] > 0 ? cg.cnt[c] : 1, 256);
         if (a64)
             gs_colour_kernel<double><<<blocks, 256, 0, s>>>(nx, ny, nz, cg, c,
