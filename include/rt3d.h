@@ -204,7 +204,7 @@ typedef struct {
                              inside the block of voxels the thread's
                              characteristics occupy, then reduced in FP64;
                              FP32 grids of at most 2^27 voxels; 96 bytes a
-                             voxel allocated on first use) */
+                             voxel while the grid has this shape) */
     int widen;            /* FP32 contribution to FP64 for the reduction: 0 the
                              conversion instruction, 1 integer moves, 2 both
                              (one characteristic per thread: alternating from

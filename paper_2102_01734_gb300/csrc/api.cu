@@ -385,17 +385,64 @@ constexpr FsShape kFsShapes[RT3D_FS_TUNE_SHAPES] = {
     {256, 1, 0, 1}, {128, 1, 1, 1}, {64, 1, 1, 1},  {128, 2, 1, 1},
     {256, 4, 1, 1}, {128, 4, 1, 1}, {64, 4, 1, 1},  {64, 1, 2, 1}};
 
-// Buffers of the four-characteristic kernel (on first use).
+// count elements, zeroed; nothing is kept where that fails
+template <typename T>
+rt3d_status alloc_zeroed(rt3d_grid *g, T **p, size_t count) {
+    T *q = nullptr;
+    TRY(g->alloc(&q, count));
+    const cudaError_t e = cudaMemsetAsync(q, 0, sizeof(T) * count, g->stream);
+    if (e != cudaSuccess) g->release(q, count);
+    CK(e);
+    *p = q;
+    return RT3D_OK;
+}
+
+// Whether device memory can be spared for buffers that a call can do without: an
+// eighth of what is free at most, and the solvers' vectors (201 of the Krylov
+// basis, the line solve's band and what else is allocated on first use: below
+// 2048 bytes a voxel) still fit.
+bool can_spare(const rt3d_grid *g, size_t bytes) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t rest = g->krylov_ready ? 0 : 2048 * (size_t)g->N;
+    return bytes <= free_b / 8 && free_b - bytes >= rest;
+}
+
+// Buffers of the four-characteristic kernel (96 bytes a voxel, on first use); both
+// or none.
 rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
     const size_t N = (size_t)g->N;
-    if (!g->pairs_t) TRY(g->alloc(&g->pairs_t, 4 * N));
     if (!g->Jrep_t) {
-        TRY(g->alloc(&g->Jrep_t, 4 * N));
-        CK(cudaMemsetAsync(g->Jrep_t, 0, sizeof(double) * 4 * N, g->stream));
+        TRY(g->alloc(&g->pairs_t, 4 * N));
+        const rt3d_status st = alloc_zeroed(g, &g->Jrep_t, 4 * N);
+        if (st != RT3D_OK) {
+            g->release(g->pairs_t, 4 * N);
+            return st;
+        }
     }
     p->pairs_t = g->pairs_t;
     p->Jrep_t = g->Jrep_t;
     return RT3D_OK;
+}
+
+// Gives them back unless the grid's shape or its Lambda* kernel uses them.
+void quad_release(rt3d_grid *g) {
+    if (g->fs_shape.rays_per_thread == 4 || g->band_t) return;
+    g->release(g->pairs_t, 4 * (size_t)g->N);
+    g->release(g->Jrep_t, 4 * (size_t)g->N);
+}
+
+// quad_setup for a call that can do without: false, with the last error's message
+// as it was, where the buffers are not to be had.
+bool quad_try(rt3d_grid *g, FsParams *p) {
+    if (!g->Jrep_t && !can_spare(g, 96 * (size_t)g->N)) return false;
+    const std::string err = g_err;
+    const bool ok = quad_setup(g, p) == RT3D_OK;
+    if (!ok) g_err = err;
+    return ok;
 }
 
 // Autotuner of the FP32 formal solution's ray-bundle shape: times one launch
@@ -404,10 +451,9 @@ rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
 // folded into g->Jfs, which the caller's launch overwrites.
 rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
-    // above 2^25 voxels the four-characteristic kernel's 96 bytes a voxel are
-    // left to the solver's vectors
-    // (nor is it a reason to fail: where its buffers do not fit it is not timed)
-    const bool four = quad_applicable(p) && g->N <= (1LL << 25) && quad_setup(g, &p) == RT3D_OK;
+    // above 2^25 voxels, or where memory is short, the four-characteristic kernel's
+    // 96 bytes a voxel are left to the solver's vectors and it is not timed
+    const bool four = quad_applicable(p) && g->N <= (1LL << 25) && quad_try(g, &p);
     float best = 0.0f;
     int pick = 0;
     for (int i = -1; i < RT3D_FS_TUNE_SHAPES; ++i) {
@@ -432,6 +478,7 @@ rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
         }
     }
     g->fs_shape = kFsShapes[pick];
+    quad_release(g);
     return RT3D_OK;
 }
 
@@ -559,26 +606,27 @@ rt3d_status run_fs_sph(rt3d_grid *g, const FsParams &base, const void *chiS, int
 }
 
 // Whether the four-characteristic kernel builds Lambda* on this grid, with its
-// buffers set up if so (320 bytes a voxel; taken once, within an eighth of the
-// free device memory: where they do not fit, the one-characteristic kernel runs).
+// buffers set up if so (320 bytes a voxel with the ones above, taken once where
+// they can be spared: elsewhere the one-characteristic kernel runs).
 bool lstar_quad(rt3d_grid *g, FsParams *p) {
     if (g->N > (1LL << 25) || !lstar_quad_applicable(*p)) return false;
+    const size_t N = (size_t)g->N;
     if (!g->band_t) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        size_t free_b = 0, total_b = 0;
-        if (cudaStreamIsCapturing(g->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-            cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
-            320 * (size_t)g->N > free_b / 8) {
+        if (cudaStreamIsCapturing(g->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
             cudaGetLastError();
             return false;
         }
-        double *q = nullptr;
-        const size_t n = 28 * (size_t)g->N;
-        if (quad_setup(g, p) != RT3D_OK || g->alloc(&q, n) != RT3D_OK) return false;
-        if (cudaMemsetAsync(q, 0, sizeof(double) * n, g->stream) != cudaSuccess) return false;
-        g->band_t = q;
+        if (!can_spare(g, (g->Jrep_t ? 224 : 320) * N) || !quad_try(g, p)) return false;
+        const std::string err = g_err;
+        if (alloc_zeroed(g, &g->band_t, 28 * N) != RT3D_OK) {
+            g_err = err;
+            quad_release(g);
+            return false;
+        }
     }
-    if (quad_setup(g, p) != RT3D_OK) return false;
+    p->pairs_t = g->pairs_t;
+    p->Jrep_t = g->Jrep_t;
     p->band_t = g->band_t;
     return true;
 }
@@ -1905,6 +1953,7 @@ rt3d_status rt3d_grid_set_fs_shape(rt3d_grid *g, const rt3d_fs_shape *shape) {
         return fail(RT3D_EINVAL, "four characteristics per thread need an FP32 Cartesian grid of "
                                  "at most 2^27 voxels");
     g->fs_shape = sh;
+    quad_release(g);
     return RT3D_OK;
 }
 
