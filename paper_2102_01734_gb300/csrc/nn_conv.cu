@@ -51,10 +51,37 @@ constexpr int kMaxHalo = 720;
 __device__ __forceinline__ unsigned smem_addr(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
-__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool valid) {
+__device__ __forceinline__ void cp_async16(unsigned dst, const bf16 *src, bool valid) {
     const int n = valid ? 16 : 0;  // 0: the 16 bytes are zero-filled, src is not read
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n)
                  : "memory");
+}
+// The same value by value, for arrays whose address is no multiple of 16.
+__device__ __forceinline__ void copy16(unsigned dst, const bf16 *src, bool valid) {
+    unsigned v[4] = {0u, 0u, 0u, 0u};
+    if (valid) {
+        const unsigned short *p = reinterpret_cast<const unsigned short *>(src);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = p[2 * i] | (unsigned)p[2 * i + 1] << 16;
+    }
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3])
+                 : "memory");
+}
+// Bits of the kernels' `wide` argument: X, the other operand (weights or dY), and
+// the outputs in pairs.
+constexpr int kWideX = 1, kWideB = 2, kWideOut = 4;
+int wide_operands(const bf16 *X, const bf16 *b) {
+    return ((reinterpret_cast<uintptr_t>(X) & 15) == 0 ? kWideX : 0) |
+           ((reinterpret_cast<uintptr_t>(b) & 15) == 0 ? kWideB : 0);
+}
+// at(i, copy) for the pieces i < n of an array, copy as its address allows. (One
+// branch for the array: in the loop it cost a training step 3 %.)
+template <int THREADS, typename F> __device__ __forceinline__ void stage(int n, bool wide, F at) {
+    if (wide)
+        for (int i = threadIdx.x; i < n; i += THREADS) at(i, cp_async16);
+    else
+        for (int i = threadIdx.x; i < n; i += THREADS) at(i, copy16);
 }
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
@@ -108,13 +135,14 @@ __device__ __forceinline__ void halo_table(int *tab, const ConvTile &t, int bx, 
     }
 }
 
+template <int THREADS>
 __device__ __forceinline__ void load_halo(unsigned dst, const int *tab, int n, const bf16 *Xs, int Ci,
-                                          int c0) {
-    for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) {
+                                          int c0, bool wide) {
+    auto at = [&](int i, auto copy) {
         const int h = i >> 1, half = i & 1, u = tab[h];
-        cp_async16(dst + halo_at(h, half), Xs + (long long)(u < 0 ? 0 : u) * Ci + c0 + 8 * half,
-                   u >= 0);
-    }
+        copy(dst + halo_at(h, half), Xs + (long long)(u < 0 ? 0 : u) * Ci + c0 + 8 * half, u >= 0);
+    };
+    stage<THREADS>(2 * n, wide, at);
 }
 
 // Halo index of tile voxel m (the halo voxel of its own position)
@@ -131,7 +159,7 @@ __global__ void __launch_bounds__(128) conv_tile_kernel(const bf16 *__restrict__
                                                         const float *__restrict__ bias,
                                                         bf16 *__restrict__ Y, float *__restrict__ Yf,
                                                         ConvTile t, int nx, int ny, int nz, int Ci,
-                                                        int relu, int sign, int vec) {
+                                                        int relu, int sign, int wide) {
     extern __shared__ __align__(128) unsigned char sm[];
     int *tab = reinterpret_cast<int *>(sm);
     const unsigned sX = smem_addr(sm) + 4 * kMaxHalo, sW = sX + 32 * kMaxHalo;
@@ -156,12 +184,11 @@ __global__ void __launch_bounds__(128) conv_tile_kernel(const bf16 *__restrict__
     const int half = lane >> 4;
     for (int c0 = 0; c0 < Ci; c0 += 16) {
         __syncthreads();
-        load_halo(sX, tab, n, Xs, Ci, c0);
-        for (int i = threadIdx.x; i < 27 * 16 * (CO / 8); i += 128) {
+        load_halo<128>(sX, tab, n, Xs, Ci, c0, wide & kWideX);
+        stage<128>(27 * 16 * (CO / 8), wide & kWideB, [&](int i, auto copy) {
             const int k = i / (CO / 8), c = i % (CO / 8);  // k = 16 tap + channel
-            cp_async16(sW + row_at<CO>(k, c), Wt + ((long long)(k >> 4) * Ci + c0 + (k & 15)) * CO + 8 * c,
-                       true);
-        }
+            copy(sW + row_at<CO>(k, c), Wt + ((long long)(k >> 4) * Ci + c0 + (k & 15)) * CO + 8 * c, true);
+        });
         cp_async_wait();
         __syncthreads();
         int d = 0;
@@ -207,7 +234,7 @@ __global__ void __launch_bounds__(128) conv_tile_kernel(const bf16 *__restrict__
                     v0 = fmaxf(v0, 0.0f);
                     v1 = fmaxf(v1, 0.0f);
                 }
-                if (vec) {
+                if (wide & kWideOut) {
                     if (Y) *reinterpret_cast<__nv_bfloat162 *>(Y + o + 8 * j) = __floats2bfloat162_rn(v0, v1);
                     if (Yf) *reinterpret_cast<float2 *>(Yf + o + 8 * j) = make_float2(v0, v1);
                 } else {
@@ -234,7 +261,8 @@ __global__ void __launch_bounds__(288) conv_wgrad_tile_kernel(const bf16 *__rest
                                                               const bf16 *__restrict__ dY,
                                                               float *__restrict__ dW,
                                                               float *__restrict__ db, ConvTile t, int S,
-                                                              int nx, int ny, int nz, int Ci, int Co) {
+                                                              int nx, int ny, int nz, int Ci, int Co,
+                                                              int wide) {
     extern __shared__ __align__(128) unsigned char sm[];
     int *tab = reinterpret_cast<int *>(sm);
     const unsigned sX = smem_addr(sm) + 4 * kMaxHalo, sY = sX + 32 * kMaxHalo;
@@ -264,16 +292,16 @@ __global__ void __launch_bounds__(288) conv_wgrad_tile_kernel(const bf16 *__rest
         __syncthreads();
         halo_table(tab, t, bx, by, bz, nx, ny, nz);
         __syncthreads();
-        load_halo(sX, tab, n, X + s * V * Ci, Ci, c0);
-        for (int i = threadIdx.x; i < P * (NC / 8); i += 288) {
+        load_halo<288>(sX, tab, n, X + s * V * Ci, Ci, c0, wide & kWideX);
+        stage<288>(P * (NC / 8), wide & kWideB, [&](int i, auto copy) {
             const int m = i / (NC / 8), c = i % (NC / 8);
             const int x = (bx << t.lx) + (m & ((1 << t.lx) - 1));
             const int y = (by << t.ly) + ((m >> t.lx) & ((1 << t.ly) - 1));
             const int z = (bz << t.lz) + (m >> (t.lx + t.ly));
             const bool in = x < nx && y < ny && z < nz;
             const long long v = in ? x + (long long)nx * (y + (long long)ny * z) : 0;
-            cp_async16(sY + row_at<NC>(m, c), dY + (s * V + v) * Co + n0 + 8 * c, in);
-        }
+            copy(sY + row_at<NC>(m, c), dY + (s * V + v) * Co + n0 + 8 * c, in);
+        });
         cp_async_wait();
         __syncthreads();
         for (int k0 = 0; k0 < P; k0 += 16) {
@@ -347,9 +375,10 @@ cudaError_t conv_go(const bf16 *X, const bf16 *Wt, const float *bias, bf16 *Y, f
     const cudaError_t e = cudaFuncSetAttribute(conv_tile_kernel<CO, MT>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     if (e != cudaSuccess) return e;
-    const int vec = (reinterpret_cast<uintptr_t>(Y) & 3) == 0 && (reinterpret_cast<uintptr_t>(Yf) & 7) == 0;
+    const bool pairs = (reinterpret_cast<uintptr_t>(Y) & 3) == 0 && (reinterpret_cast<uintptr_t>(Yf) & 7) == 0;
     conv_tile_kernel<CO, MT><<<dim3(t.tiles(), S), 128, shm, s>>>(X, Wt, bias, Y, Yf, t, nx, ny, nz, Ci,
-                                                                  relu ? 1 : 0, sign, vec);
+                                                                  relu ? 1 : 0, sign,
+                                                                  wide_operands(X, Wt) | (pairs ? kWideOut : 0));
     return cudaGetLastError();
 }
 
@@ -377,8 +406,8 @@ cudaError_t wgrad_go(const bf16 *X, const bf16 *dY, float *dW, float *db, int S,
     if (e != cudaSuccess) return e;
     const long long all = (long long)t.tiles() * S;
     const int gx = (int)std::max(1LL, std::min(all, (long long)(2 * sms + parts - 1) / parts));
-    conv_wgrad_tile_kernel<NC><<<dim3(gx, Ci / 16, Co / NC), 288, shm, s>>>(X, dY, dW, db, t, S, nx, ny,
-                                                                            nz, Ci, Co);
+    conv_wgrad_tile_kernel<NC><<<dim3(gx, Ci / 16, Co / NC), 288, shm, s>>>(
+        X, dY, dW, db, t, S, nx, ny, nz, Ci, Co, wide_operands(X, dY));
     return cudaGetLastError();
 }
 
