@@ -9,10 +9,11 @@
  * Convolutions are 3x3x3, periodic in x and y and zero-padded in z. Weights
  * are Wt[d][Ci][Co] (BF16) with d = (dz+1)*9 + (dy+1)*3 + (dx+1); the data
  * gradient uses the transposed copy WT[d][Co][Ci]. Gradient accumulators are
- * FP32 and must be zeroed by the caller. All pointers are device memory aligned
- * to their type (16-byte addresses are the fast ones); all work is issued on `stream` (NULL: legacy stream) without synchronising.
- * Every call returns RT3D_OK, RT3D_EINVAL for unsupported sizes, or
- * RT3D_ECUDA (message in rt3d_last_error()).
+ * FP32, must be zeroed by the caller and are added to atomically (several streams
+ * may share one). All pointers are device memory aligned to their type (16-byte
+ * addresses are the fast ones); all work is issued on `stream` (NULL: legacy
+ * stream) without synchronising. Every call returns RT3D_OK, RT3D_EINVAL for
+ * unsupported sizes, or RT3D_ECUDA (message in rt3d_last_error()).
  */
 #ifndef RT3D_NN_H
 #define RT3D_NN_H

@@ -44,6 +44,17 @@ template <int W, typename T> __device__ __forceinline__ void vstore(T *p, const 
     *reinterpret_cast<Vec<T, W> *>(p) = v;
 }
 
+// *p += v, each value atomically: several streams may accumulate into one buffer
+template <int W> __device__ __forceinline__ void vadd(float *p, const Vec<float, W> &v) {
+    if constexpr (W == 8) {
+        atomicAdd(reinterpret_cast<float4 *>(p), make_float4(v.v[0], v.v[1], v.v[2], v.v[3]));
+        atomicAdd(reinterpret_cast<float4 *>(p) + 1, make_float4(v.v[4], v.v[5], v.v[6], v.v[7]));
+    } else {
+        static_assert(W == 1, "one value or eight");
+        atomicAdd(p, v.v[0]);
+    }
+}
+
 // dYpre = dY * (Y > 0)
 template <int W, typename I>
 __global__ void relu_bwd_kernel(const bf16 *dY, const bf16 *Y, bf16 *out, I n) {
@@ -115,7 +126,7 @@ __global__ void pool_bwd_kernel(const bf16 *dP, float *dX32, Geo g, Geo p, int C
         const int px[2] = {q.x / 2, p.nx - 1}, py[2] = {q.y / 2, p.ny - 1};
         const int ex = (g.nx & 1) && q.x == 0 ? 2 : 1, ey = (g.ny & 1) && q.y == 0 ? 2 : 1;
         float *o = dX32 + (s * (long long)V + v) * C + c;
-        Vec<float, W> acc = vload<W>(o);
+        Vec<float, W> acc{};
         for (int b = 0; b < ey; ++b)
             for (int a = 0; a < ex; ++a) {
                 const Vec<bf16, W> d = vload<W>(
@@ -123,7 +134,7 @@ __global__ void pool_bwd_kernel(const bf16 *dP, float *dX32, Geo g, Geo p, int C
 #pragma unroll
                 for (int k = 0; k < W; ++k) acc.v[k] += __bfloat162float(d.v[k]) * 0.125f;
             }
-        vstore<W>(o, acc);
+        vadd<W>(o, acc);
     }
 }
 
@@ -154,7 +165,7 @@ __global__ void up_bwd_kernel(const bf16 *dU, float *dX32, Geo g, Geo p, int C, 
         split<W>(i, C, Vp, c, s, vp);
         const int3 q = coords(vp, p);
         float *o = dX32 + (s * (long long)Vp + vp) * C + c;
-        Vec<float, W> acc = vload<W>(o);
+        Vec<float, W> acc{};
         for (int z = 2 * q.z; z < min(2 * q.z + 2, g.nz); ++z)
             for (int y = 2 * q.y; y < min(2 * q.y + 2, g.ny); ++y)
                 for (int x = 2 * q.x; x < min(2 * q.x + 2, g.nx); ++x) {
@@ -163,7 +174,7 @@ __global__ void up_bwd_kernel(const bf16 *dU, float *dX32, Geo g, Geo p, int C, 
 #pragma unroll
                     for (int k = 0; k < W; ++k) acc.v[k] += __bfloat162float(d.v[k]);
                 }
-        vstore<W>(o, acc);
+        vadd<W>(o, acc);
     }
 }
 
