@@ -218,7 +218,8 @@ class UNet:
         s1s, s2s, s3s = shape, half(shape), half(half(shape))
         # one zeroed allocation for all accumulators (a fill instead of 22)
         params = [*self.W32.items(), *self.b32.items()]
-        parts = torch.zeros(self.n_params(), device=self.dev).split([p.numel() for _, p in params])
+        parts = torch.zeros(self.n_params(), dtype=torch.float32, device=self.dev).split(
+            [p.numel() for _, p in params])
         views = [z.view(p.shape) for z, (_, p) in zip(parts, params)]
         self.gW = {n: z for n, z in zip(self.W32, views)}
         self.wgrad_inputs = {}
