@@ -655,7 +655,7 @@ rt3d_status run_fs(rt3d_grid *g, const FsParams &base, bool fp64, bool with_lsta
     if (lquad) CK(launch_fs_lstar_quad(p, g->parab, g->stream));
     else if (fast && fp64) CK(launch_fs64_fast(p, g->parab, g->stream));
     else if (fast) CK(launch_fs_fast(p, g->parab, g->fs_shape, g->stream));
-    else CK(launch_fs(p, fp64, g->parab, with_lstar, g->stream));
+    else CK(launch_fs_lstar(p, fp64, g->parab, g->stream));
     CK(cudaEventRecord(g->ev1, g->stream));
     g->ev_pending = fp64 ? 1 : (with_lstar ? 3 : 0);
     if (!fp64 && with_lstar) ++g->fs_lstar32;
@@ -2478,7 +2478,7 @@ rt3d_status rt3d_solve_batched(rt3d_grid *g, int nl, const double *chi, const do
         p.homogeneous = 1;
         CK(cudaMemsetAsync(g->Jfs, 0, sizeof(double) * N, s));
         CK(cudaMemsetAsync(g->lstar, 0, sizeof(double) * 27 * N, s));
-        CKL(launch_fs(p, false, g->parab, true, s));
+        CKL(launch_fs_lstar(p, false, g->parab, s));
         CKL(launch_os_prep(g->nx, g->ny, g->nz, g->lstar, g->beps + l * N, g->ba + l * os_coef_count((long long)N),
                            false, g->binv + l * N, s, g->per));
         ++bs.fs_lambda32;

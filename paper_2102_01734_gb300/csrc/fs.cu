@@ -128,7 +128,7 @@ __device__ __forceinline__ int rep_of(uint32_t c, int x0, int y0, int nx, int ny
 // voxels, 128 angles 3.24 ms with the library's exp, divisions and an 18-term
 // series, 1.98 ms with interval64_w and recip64; parabolic 4.98 -> 3.23 ms. Error of
 // Lambda* against 64 bits 7.8e-16 -> 7.1e-16).
-template <typename R, bool PARAB, bool LSTAR>
+template <typename R, bool PARAB>
 __global__ void __launch_bounds__(128) fs_kernel(FsParams p) {
     using R2 = typename V2<R>::T;
     __shared__ unsigned long long tab[64];
@@ -191,21 +191,19 @@ __global__ void __launch_bounds__(128) fs_kernel(FsParams p) {
         I = f.E * I + al * S_p + bg * S_c + ga * (S_n - S_c);
         const R c = __ldg(cw + k);
         atomicAdd(p.J + v, red_value(c * I));
-        if (LSTAR) {
-            // ring[i] = dI_k / dS_{k-7+i}
+        // ring[i] = dI_k / dS_{k-7+i}
 #pragma unroll
-            for (int i = 0; i < kWin - 1; ++i) ring[i] = f.E * ring[i + 1];
-            const R be = bg - ga;
-            if (k == 0) ring[7] += al;  // S_{-1} = S_0 at the entry point
-            else ring[6] += al;
-            ring[7] += be;
-            ring[8] = ga;
-            const uint64_t wc = __ldg(reinterpret_cast<const unsigned long long *>(p.win + t0 + k));
+        for (int i = 0; i < kWin - 1; ++i) ring[i] = f.E * ring[i + 1];
+        const R be = bg - ga;
+        if (k == 0) ring[7] += al;  // S_{-1} = S_0 at the entry point
+        else ring[6] += al;
+        ring[7] += be;
+        ring[8] = ga;
+        const uint64_t wc = __ldg(reinterpret_cast<const unsigned long long *>(p.win + t0 + k));
 #pragma unroll
-            for (int i = 0; i < kWin; ++i) {
-                const unsigned dc = (unsigned)(wc >> (5 * i)) & 31u;
-                if (dc != kWinNone) atomicAdd(p.lstar + (long long)dc * N + v, red_value(c * ring[i]));
-            }
+        for (int i = 0; i < kWin; ++i) {
+            const unsigned dc = (unsigned)(wc >> (5 * i)) & 31u;
+            if (dc != kWinNone) atomicAdd(p.lstar + (long long)dc * N + v, red_value(c * ring[i]));
         }
         chil_p = chil_c;
         chil_c = chil_n;
@@ -909,11 +907,11 @@ __global__ void fold_kernel(int nx, int ny, int nz, double *__restrict__ Jrep,
     }
 }
 
-template <typename R, bool PARAB, bool LSTAR>
+template <typename R, bool PARAB>
 cudaError_t launch_t(const FsParams &p, cudaStream_t s) {
     const int threads = 128;
     dim3 grid((p.nx * p.ny + threads - 1) / threads, p.nangles);
-    fs_kernel<R, PARAB, LSTAR><<<grid, threads, 0, s>>>(p);
+    fs_kernel<R, PARAB><<<grid, threads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -1032,13 +1030,9 @@ cudaError_t launch_fold(int nx, int ny, int nz, double *Jrep, double *J, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_fs(const FsParams &p, bool fp64, bool parabolic, bool lstar, cudaStream_t s) {
-    if (fp64) {
-        if (parabolic) return lstar ? launch_t<double, true, true>(p, s) : launch_t<double, true, false>(p, s);
-        return lstar ? launch_t<double, false, true>(p, s) : launch_t<double, false, false>(p, s);
-    }
-    if (parabolic) return lstar ? launch_t<float, true, true>(p, s) : launch_t<float, true, false>(p, s);
-    return lstar ? launch_t<float, false, true>(p, s) : launch_t<float, false, false>(p, s);
+cudaError_t launch_fs_lstar(const FsParams &p, bool fp64, bool parabolic, cudaStream_t s) {
+    if (fp64) return parabolic ? launch_t<double, true>(p, s) : launch_t<double, false>(p, s);
+    return parabolic ? launch_t<float, true>(p, s) : launch_t<float, false>(p, s);
 }
 
 }  // namespace rt3d

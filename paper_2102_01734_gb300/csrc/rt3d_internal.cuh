@@ -143,7 +143,9 @@ struct TraceParams {
 
 // Launchers (return the launch status).
 cudaError_t launch_trace(const TraceParams &p, cudaStream_t s);
-cudaError_t launch_fs(const FsParams &p, bool fp64, bool parabolic, bool lstar, cudaStream_t s);
+// formal solution with Lambda*, one characteristic per thread: into p.J and p.lstar
+// (zeroed by the caller)
+cudaError_t launch_fs_lstar(const FsParams &p, bool fp64, bool parabolic, cudaStream_t s);
 // Ray-bundle shape of the FP32 formal solution without Lambda* (the same
 // fields as the public rt3d_fs_shape).
 struct FsShape {
@@ -163,6 +165,8 @@ bool quad_applicable(const FsParams &p);
 // and p.lstar (zeroed by the caller); whether it can run on these parameters and
 // fills the device
 bool lstar_quad_applicable(const FsParams &p);
+// formal solution with Lambda*, one characteristic per thread: into p.J and p.lstar
+// (zeroed by the caller)
 cudaError_t launch_fs_lstar_quad(const FsParams &p, bool parabolic, cudaStream_t s);
 // the four-characteristic kernel's step records from the template
 cudaError_t launch_quad_rec(const Template &t, int nx, int ny, float4 *rec4, cudaStream_t s);
