@@ -77,8 +77,9 @@ def host(tmp_path_factory):
             f.write(text)
     subprocess.run([build.nvcc(), *build._flags(["-I", build.SRC_DIR]), "-c", paths["call.cu"], "-o", paths["call.o"]],
                    check=True)
-    subprocess.run(["g++", "-shared", "-fPIC", "-o", paths["host.so"], paths["runtime.cpp"], paths["call.o"],
-                    os.path.join(build.OUT_DIR, "ali.o")], check=True)
+    # -Bsymbolic: this runtime also where the process has loaded the real one
+    subprocess.run(["g++", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-o", paths["host.so"], paths["runtime.cpp"],
+                    paths["call.o"], os.path.join(build.OUT_DIR, "ali.o")], check=True)
     lib = ctypes.CDLL(paths["host.so"])
     lib.launches.restype = ctypes.c_char_p
     return lib
