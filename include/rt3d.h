@@ -292,7 +292,8 @@ rt3d_status rt3d_fs_tune_shape(int i, rt3d_fs_shape *out);
  * default for a new grid): every candidate of rt3d_fs_tune_shape that the
  * grid supports is launched once on that call's input, timed with CUDA
  * events on the grid's stream, and the fastest is kept (an unsupported
- * candidate records 0 ms in rt3d_grid_info). The result does not depend on the shape beyond
+ * candidate records 0 ms in rt3d_grid_info, and so do candidates that shapes timed
+ * before them leave no chance). The result does not depend on the shape beyond
  * FP64 reduction order (both widenings are exact for normal FP32 values;
  * integer widening maps an FP32 zero or subnormal contribution to at most
  * 1.2e-38 in magnitude). RT3D_EINVAL for a shape outside the ranges of
