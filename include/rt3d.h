@@ -292,11 +292,14 @@ rt3d_status rt3d_fs_tune_shape(int i, rt3d_fs_shape *out);
  * default for a new grid): every candidate of rt3d_fs_tune_shape that the
  * grid supports is launched once on that call's input, timed with CUDA
  * events on the grid's stream, and the fastest is kept (an unsupported
- * candidate records 0 ms in rt3d_grid_info, and so do candidates that shapes timed
- * before them leave no chance). The result does not depend on the shape beyond
- * FP64 reduction order (both widenings are exact for normal FP32 values;
- * integer widening maps an FP32 zero or subnormal contribution to at most
- * 1.2e-38 in magnitude). RT3D_EINVAL for a shape outside the ranges of
+ * candidate records 0 ms in rt3d_grid_info, and so do one whose buffers memory
+ * cannot spare and those that shapes timed before them leave no chance). Shapes
+ * differ in the FP32 rounding of a step and of the sums (about 2e-8 of J) and in
+ * the FP64 reduction order; both widenings are exact for normal FP32 values,
+ * integer widening maps an FP32 zero or subnormal contribution to at most 1.2e-38
+ * in magnitude. With two or four characteristics per thread the parabolic term
+ * fades out below an optical depth of 1e-15 a step (1e-37 with one).
+ * RT3D_EINVAL for a shape outside the ranges of
  * rt3d_fs_shape, or four characteristics per thread on a grid that does
  * not support them. */
 rt3d_status rt3d_grid_set_fs_shape(rt3d_grid *grid, const rt3d_fs_shape *shape);
@@ -326,7 +329,12 @@ rt3d_status rt3d_grid_sph_ray(const rt3d_grid *grid, int angle, int index, int *
  * chi > 0 (per unit length) and S: double[N]. J_out: double[N] (written).
  * lstar_out: nullable double[27][N]; when given, the passage-local Lambda*
  * band (Sec. 4, "non-local Lambda*") is built as well. bc: nullable (zero
- * incoming intensity). */
+ * incoming intensity).
+ * Where enough characteristics fill the device, FP32 Lambda* comes from a kernel
+ * that needs 320 bytes a voxel, taken at the first such call and held by the grid.
+ * They are taken only if they are within an eighth of the free device memory and
+ * leave the solvers' vectors (2 kB a voxel): elsewhere the general kernel runs, whose
+ * result differs by FP32 rounding. Several grids each hold their own. */
 rt3d_status rt3d_formal_solution(rt3d_grid *grid, const double *chi, const double *S,
                                  const rt3d_bc *bc, double *J_out, double *lstar_out);
 

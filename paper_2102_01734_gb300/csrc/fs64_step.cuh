@@ -147,7 +147,8 @@ __device__ __forceinline__ unsigned long long exp_fixed64(double u, const unsign
     k = n >> 6;
     return __umul64hi(tab[n & 63], (1ULL << 63) + (unsigned long long)(P >> 1));
 }
-// 1 - e^-u and e^-u, rounded once
+// 1 - e^-u and e^-u, rounded once: within 2.4 2^-53 of themselves (the table's
+// rounding, the cut of the series and the last rounding)
 __device__ __forceinline__ double one_minus_exp64(double u, const unsigned long long *tab) {
     int k;
     const unsigned long long E = exp_fixed64(u, tab, k);

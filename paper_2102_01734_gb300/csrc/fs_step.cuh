@@ -1,6 +1,7 @@
-// Per-point arithmetic of the FP32 formal solution without Lambda*, shared
-// by the single-problem kernel (fs.cu) and the batched-wavelength kernel
-// (batch.cu). The interval functions and the update follow the construction
+// Per-point arithmetic of the FP32 formal solutions: with one, two and four
+// characteristics a thread, and with the weights of Lambda* (fs.cu); one
+// characteristic a thread also serves the batched wavelengths (batch.cu) and the
+// shell (sph.cu). The interval functions and the update follow the construction
 // documented at the top of fs.cu (Olson & Kunasz 1987 weights with the
 // limited parabola; the update in difference form).
 #pragma once
@@ -149,11 +150,11 @@ struct RayP {
 };
 
 // One point of a pair of characteristics, given c, the pair-packed (chi, S)
-// of the next point, and hl, the pair (l/2, l/2) of its chord: the update of
-// fast_step on both characteristics (the parabolic correction always
+// of the next point, and hl, the pair (l/2, l/2) of its chord: the update in
+// difference form on both characteristics (the parabolic correction always
 // evaluated, its blend weight 0 where the linear form applies), and the
 // advance to the next point. Returns the intensities at the current point.
-// The two reciprocals of the scalar step come from one: with
+// The two divisions share one reciprocal: with
 // X = wf (u + wf), 1/wf = (u + wf)/X and u/(u + wf) = u wf/X, where wf is
 // the next interval floored at 1e-15 (so X >= 1e-30 stays a normal FP32
 // number; a zero-opacity interval gets q = 0 or blend weight 0).

@@ -6,8 +6,8 @@
 // Activations are BF16, channel-last [S][V][C] (S samples, V = nx*ny*nz
 // voxels, x fastest, C a multiple of 16). Convolutions are 3x3x3, periodic in
 // x and y, zero-padded in z (the geometry of the radiative-transfer box),
-// computed as implicit GEMMs on the tensor cores: BF16 operands, FP32
-// accumulation (nvcuda::wmma 16x16x16 tiles). Weights are stored per
+// computed as implicit GEMMs on the tensor cores (nn_conv.cu): BF16 operands,
+// FP32 accumulation, mma.sync m16n8k16. Weights are stored per
 // offset d = (dz+1)*9 + (dy+1)*3 + (dx+1) as Wt[d][Ci][Co] (BF16), with an
 // FP32 master copy for the optimiser.
 #include <cuda_bf16.h>
