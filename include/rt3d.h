@@ -224,7 +224,7 @@ typedef struct {
     long long device_bytes;   /* device memory held by the grid */
     rt3d_fs_shape fs_shape;   /* ray-bundle shape of the FP32 formal solution
                                  without Lambda* (block 0: not chosen yet) */
-    float fs_tune_ms[RT3D_FS_TUNE_SHAPES]; /* kernel time of each candidate
+    float fs_tune_ms[RT3D_FS_TUNE_SHAPES]; /* device time of each candidate
                                  shape (rt3d_fs_tune_shape order) at the last
                                  autotuning; 0 if not tuned */
     int sm_count;             /* streaming multiprocessors of the grid's device

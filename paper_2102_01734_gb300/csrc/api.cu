@@ -472,9 +472,9 @@ rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
         }
         CK(cudaEventRecord(g->ev0, g->stream));
         CK(launch_fs_fast(p, g->parab, kFsShapes[c], g->stream));
-        CK(cudaEventRecord(g->ev1, g->stream));
         CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream,
                        kFsShapes[c].rays_per_thread == 4 ? g->Jrep_t : nullptr));
+        CK(cudaEventRecord(g->ev1, g->stream));  // the fold of two arrays takes longer
         g->launches += 2;
         CK(cudaEventSynchronize(g->ev1));
         float ms = 0.0f;
