@@ -451,22 +451,25 @@ bool quad_try(rt3d_grid *g, FsParams *p) {
 // folded into g->Jfs, which the caller's launch overwrites.
 rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
-    // above 2^25 voxels, or where memory is short, the four-characteristic kernel's
-    // 96 bytes a voxel are left to the solver's vectors and it is not timed
-    const bool four = quad_applicable(p) && g->N <= (1LL << 25) && quad_try(g, &p);
     // The first one-characteristic shape, the others, then the rest of the
-    // one-characteristic ones: these are within 8 % of the first (33^3 to 129^3), so
-    // where another shape is 15 % ahead of it and a launch takes long enough to
-    // matter (0.2 ms) they are left out (four launches of 52 ms at 129^3).
+    // one-characteristic ones. Where a launch takes long enough to matter (0.2 ms),
+    // shapes without a chance are left out: the four-characteristic kernel below two
+    // waves of its groups (it is behind up to 1.75 waves and ahead from 2.7 on), and
+    // the rest where another shape is 10 % ahead of the first, as they are within 8 %
+    // of it (33^3 to 129^3; four launches of 52 ms at 129^3).
     constexpr int order[] = {-1, 0, 3, 4, 5, 6, 1, 2, 7};
     static_assert(sizeof order / sizeof order[0] == RT3D_FS_TUNE_SHAPES + 1, "every shape once");
     float best = 0.0f;
     int pick = 0;
     for (int i : order) {
         const int c = i < 0 ? 0 : i;
-        const bool behind = c > 0 && kFsShapes[c].rays_per_thread == 1 && g->fs_tune_ms[0] > 0.2f &&
-                            best < 0.85f * g->fs_tune_ms[0];
-        if (behind || (kFsShapes[c].rays_per_thread == 4 && !four)) {
+        const bool longer = c > 0 && g->fs_tune_ms[0] > 0.2f;
+        const bool behind = longer && kFsShapes[c].rays_per_thread == 1 && best < 0.9f * g->fs_tune_ms[0];
+        // above 2^25 voxels, or where memory is short, the four-characteristic kernel's
+        // 96 bytes a voxel are left to the solver's vectors
+        const bool four = kFsShapes[c].rays_per_thread == 4;
+        if (behind || (four && (!quad_applicable(p) || g->N > (1LL << 25) ||
+                                (longer && quad_waves(p) < 2.0) || !quad_try(g, &p)))) {
             g->fs_tune_ms[c] = 0.0f;  // not timed
             continue;
         }
