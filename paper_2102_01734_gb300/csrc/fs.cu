@@ -335,12 +335,12 @@ __global__ void __launch_bounds__(256) fs_pair_kernel(FsParams p) {
 // of the other axis, so that loads and reductions stay contiguous: the angles
 // that step along x more than along y run on arrays with x and y exchanged
 // (pairs_t, Jrep_t, offsets of their records).
-// Measured against the pair kernel: 129^3, 2048 angles 46.2 -> 38.4 ms (7.6e11
-// segments/s), 97^3, 512 angles 4.29 -> 3.45 ms, 65^3 1.35 -> 1.21 ms; at 33^3,
-// 128 angles 0.165 against 0.110 ms (one per thread), where the longest
+// Measured against the pair kernel: 129^3, 2048 angles 45.8 -> 38.1 ms (7.7e11
+// segments/s), 97^3, 512 angles 4.23 -> 3.42 ms, 65^3 1.35 -> 1.18 ms; at 33^3,
+// 128 angles 0.166 against 0.088 ms (one per thread), where the longest
 // characteristic's latency counts. Bound by FP32 issue: 80 warp instructions per
 // point of two warps' worth of segments (99 without the votes and the sums), 35
-// of them FP32, 71 % of the issue slots at 24 warps a SM (80 registers).
+// of them FP32, 66 % of the issue slots at 24 warps a SM (80 registers).
 // A sum holds at most the contributions of the rows that pass its voxel at
 // successive points. Rows past the face (its last quad) are integrated like the
 // others; their sums are never reduced and never move into an existing row.
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(256, 3) fs_quad_kernel(FsParams p) {
 // 27 planes and J), added to the others afterwards (band_merge_kernel, 0.16 ms at
 // 97^3). 154 registers: six blocks of 64 a SM without spills; four blocks of 128
 // spill and are no faster. With both kernels and 512 angles: 65 x 65 x 257 27.4 ->
-// 22.5 ms, 97^3 21.2 -> 17.2 ms; at 65 x 65 x 257 the L2's atomic input is 73 %
+// 22.6 ms, 97^3 21.2 -> 17.2 ms; at 65 x 65 x 257 the L2's atomic input is 72 %
 // busy, issue 54 %. Error of Lambda* against 64 bits at 65^3: 6.83e-9 -> 6.80e-9 (interval
 // functions from the 9-term series, alpha without cancellation: with the
 // polynomials of the kernel above and e0 - a it was 7.6e-9).

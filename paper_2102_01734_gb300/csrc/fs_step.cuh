@@ -472,9 +472,9 @@ __device__ __forceinline__ void quad_last_w(RayN &s, WeightsN &w) {
 // instruction stream, and only I + e0 (Sp - I) + B remains in sequence. The
 // chain a point waits for is halved, which is what counts where few warps are
 // left (small grids, scattered rays). Against the point-by-point form (one
-// packed lane unused): box 33^3, 128 angles 107 -> 93 us, shell 65 x 33 x 65,
-// 512 angles 2.17 -> 2.08 ms, eight batched wavelengths on 33^3 134 -> 127 ms a
-// solve; large boxes gain nothing (97^3 4.74 -> 4.89 ms), but they run four
+// packed lane unused): box 33^3, 128 angles 107 -> 88 us, shell 65 x 33 x 65,
+// 512 angles 2.17 -> 2.07 ms, eight batched wavelengths on 33^3 134 -> 127 ms a
+// solve; large boxes gain nothing (97^3 4.74 ms both), but they run four
 // characteristics a thread.
 struct RayT {
     float I, u, hc, Sp, Sc;

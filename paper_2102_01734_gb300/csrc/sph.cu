@@ -604,9 +604,12 @@ namespace {
 // fall on nearby cells (21 % faster than ordering by ray length, which matches
 // trip counts but scatters a warp over the shell); contributions widened by
 // integer moves (the FP64 pipe stays free) and reduced in FP64 at the
-// replicated index (folded afterwards). Bound by the L2: nearly every segment's
-// reduction is a sector of its own. Loading a point ahead cost 1 to 4 %: the
-// lanes of a warp run rays of different lengths.
+// replicated index (folded afterwards). What bounds it is the latency of the
+// records and gathers in warps that are mostly empty: a warp runs until its
+// longest ray ends, 12 of 32 lanes are active on average, an instruction waits 23
+// issue slots for loads, and issue (28 %), L2 atomic input (24 %) and DRAM (the
+// records, 1.6 TB/s) are far from busy (33 x 17 x 33 cells, 512 angles, 0.31 ms).
+// Loading a point ahead cost 1 to 4 %.
 template <bool PARAB>
 __global__ void __launch_bounds__(128) sph_fs_fast_kernel(SphFsParams p, double *__restrict__ Jrep) {
     const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
