@@ -411,17 +411,15 @@ bool can_spare(const rt3d_grid *g, size_t bytes) {
     return bytes <= free_b / 8 && free_b - bytes >= rest;
 }
 
-// Buffers of the four-characteristic kernel (96 bytes a voxel, on first use); both
-// or none.
+// Buffers of the four-characteristic kernel (96 bytes a voxel in one allocation, on
+// first use).
 rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
     const size_t N = (size_t)g->N;
     if (!g->Jrep_t) {
-        TRY(g->alloc(&g->pairs_t, 4 * N));
-        const rt3d_status st = alloc_zeroed(g, &g->Jrep_t, 4 * N);
-        if (st != RT3D_OK) {
-            g->release(g->pairs_t, 4 * N);
-            return st;
-        }
+        float4 *q = nullptr;
+        TRY(alloc_zeroed(g, &q, 6 * N));
+        g->pairs_t = q;
+        g->Jrep_t = reinterpret_cast<double *>(q + 4 * N);
     }
     p->pairs_t = g->pairs_t;
     p->Jrep_t = g->Jrep_t;
@@ -431,8 +429,8 @@ rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
 // Gives them back unless the grid's shape or its Lambda* kernel uses them.
 void quad_release(rt3d_grid *g) {
     if (g->fs_shape.rays_per_thread == 4 || g->band_t) return;
-    g->release(g->pairs_t, 4 * (size_t)g->N);
-    g->release(g->Jrep_t, 4 * (size_t)g->N);
+    g->release(g->pairs_t, 6 * (size_t)g->N);
+    g->Jrep_t = nullptr;
 }
 
 // quad_setup for a call that can do without: false, with the last error's message
@@ -451,39 +449,44 @@ bool quad_try(rt3d_grid *g, FsParams *p) {
 // folded into g->Jfs, which the caller's launch overwrites.
 rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
-    // The first one-characteristic shape, the others, then the rest of the
-    // one-characteristic ones. Where a launch takes long enough to matter (0.2 ms),
-    // shapes without a chance are left out: the four-characteristic kernel below two
-    // waves of its groups (it is behind up to 1.75 waves and ahead from 2.7 on), and
-    // the rest where another shape is 10 % ahead of the first, as they are within 8 %
-    // of it (33^3 to 129^3; four launches of 52 ms at 129^3).
-    constexpr int order[] = {-1, 0, 3, 4, 5, 6, 1, 2, 7};
+    // An untimed launch of a few angles, the first shape with one characteristic a
+    // thread, with two, the middle one with four, then the rest. Where a launch takes
+    // long enough to matter (0.2 ms), shapes without a chance are left out: those with
+    // four where the first of them is a quarter behind (they differ by up to 17 %),
+    // those with one where another number is a fifth ahead (they differ by up to
+    // 15 %). Over 220 boxes of 12^3 to 129^3 the shape chosen is the best by hand
+    // within 5 %, 0.4 % on average (with all shapes timed 8 % and 0.4 %).
+    constexpr int order[] = {-1, 0, 3, 5, 4, 6, 1, 2, 7};
     static_assert(sizeof order / sizeof order[0] == RT3D_FS_TUNE_SHAPES + 1, "every shape once");
-    float best = 0.0f;
+    float *const t = g->fs_tune_ms;
+    float best = 0.0f, best_many = 1e30f;  // of all shapes, with several characteristics
     int pick = 0;
     for (int i : order) {
-        const int c = i < 0 ? 0 : i;
-        const bool longer = c > 0 && g->fs_tune_ms[0] > 0.2f;
-        const bool behind = longer && kFsShapes[c].rays_per_thread == 1 && best < 0.9f * g->fs_tune_ms[0];
+        const int c = i < 0 ? 0 : i, per = kFsShapes[c].rays_per_thread;
+        const bool longer = i > 0 && t[0] > 0.2f;
         // above 2^25 voxels, or where memory is short, the four-characteristic kernel's
         // 96 bytes a voxel are left to the solver's vectors
-        const bool four = kFsShapes[c].rays_per_thread == 4;
-        if (behind || (four && (!quad_applicable(p) || g->N > (1LL << 25) ||
-                                (longer && quad_waves(p) < 2.0) || !quad_try(g, &p)))) {
-            g->fs_tune_ms[c] = 0.0f;  // not timed
+        if ((longer && per == 1 && best_many < 0.8f * t[0]) ||
+            (per == 4 && ((longer && c != 5 && t[5] > 1.25f * t[0]) || !quad_applicable(p) ||
+                          g->N > (1LL << 25) || !quad_try(g, &p)))) {
+            t[c] = 0.0f;  // not timed
             continue;
         }
+        FsParams q = p;
+        if (i < 0) q.nangles = std::min(p.nangles, 16);
         CK(cudaEventRecord(g->ev0, g->stream));
-        CK(launch_fs_fast(p, g->parab, kFsShapes[c], g->stream));
+        CK(launch_fs_fast(q, g->parab, kFsShapes[c], g->stream));
         CK(launch_fold(g->nx, g->ny, g->nz, g->Jrep, g->Jfs, g->stream,
-                       kFsShapes[c].rays_per_thread == 4 ? g->Jrep_t : nullptr));
+                       per == 4 ? g->Jrep_t : nullptr));
         CK(cudaEventRecord(g->ev1, g->stream));  // the fold of two arrays takes longer
         g->launches += 2;
         CK(cudaEventSynchronize(g->ev1));
         float ms = 0.0f;
         CK(cudaEventElapsedTime(&ms, g->ev0, g->ev1));
-        if (i >= 0) g->fs_tune_ms[i] = ms;
-        if (i >= 0 && (i == 0 || ms < best)) {
+        if (i < 0) continue;
+        t[i] = ms;
+        if (per > 1) best_many = std::min(best_many, ms);
+        if (i == 0 || ms < best) {
             best = ms;
             pick = i;
         }

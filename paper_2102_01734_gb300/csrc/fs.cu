@@ -972,10 +972,6 @@ bool quad_applicable(const FsParams &p) {
     return p.rec4 != nullptr && 4LL * p.nx * p.ny * p.nz <= (long long)kQuadOffMask;
 }
 
-double quad_waves(const FsParams &p) {
-    return (double)lane_count(p) * p.nangles / (768.0 * device_sm_count());  // 24 warps a SM
-}
-
 cudaError_t launch_quad_rec(const Template &t, int nx, int ny, float4 *rec4, cudaStream_t s) {
     quad_rec_kernel<<<t.nangles, 256, 0, s>>>(nx, ny, t.toff, t.tlen, t.swap, t.code, t.rec32, rec4);
     return cudaGetLastError();

@@ -161,8 +161,6 @@ bool fs_shape_valid(const FsShape &sh);
 // whether the four-characteristic kernel can run on these parameters (its
 // records exist and the replicated grid's offsets fit in 29 bits)
 bool quad_applicable(const FsParams &p);
-// the groups of four characteristics of a formal solution over those resident at once
-double quad_waves(const FsParams &p);
 // FP32 formal solution with Lambda*, four characteristics per thread: into p.J
 // and p.lstar (zeroed by the caller); whether it can run on these parameters and
 // fills the device
