@@ -204,7 +204,8 @@ typedef struct {
                              inside the block of voxels the thread's
                              characteristics occupy, then reduced in FP64;
                              FP32 grids of at most 2^27 voxels; 96 bytes a
-                             voxel while the grid has this shape) */
+                             voxel while the grid has this shape, below 16 MB
+                             from the first use on) */
     int widen;            /* FP32 contribution to FP64 for the reduction: 0 the
                              conversion instruction, 1 integer moves, 2 both
                              (one characteristic per thread: alternating from

@@ -426,9 +426,10 @@ rt3d_status quad_setup(rt3d_grid *g, FsParams *p) {
     return RT3D_OK;
 }
 
-// Gives them back unless the grid's shape or its Lambda* kernel uses them.
+// Gives them back unless the grid's shape or its Lambda* kernel uses them, or they
+// are below 16 MB (the free takes 0.1 ms, a tenth of a small grid's first call).
 void quad_release(rt3d_grid *g) {
-    if (g->fs_shape.rays_per_thread == 4 || g->band_t) return;
+    if (g->fs_shape.rays_per_thread == 4 || g->band_t || 96 * g->N < (16LL << 20)) return;
     g->release(g->pairs_t, 6 * (size_t)g->N);
     g->Jrep_t = nullptr;
 }
@@ -450,8 +451,8 @@ bool quad_try(rt3d_grid *g, FsParams *p) {
 rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     TRY(collect_events(g));
     // An untimed launch of a few angles, the first shape with one characteristic a
-    // thread, with two, the middle one with four, then the rest. Where a launch takes
-    // long enough to matter (0.2 ms), shapes without a chance are left out: those with
+    // thread, with two, the middle one with four, then the rest. Where even the
+    // fastest so far takes long enough to matter (0.2 ms), shapes without a chance are left out: those with
     // four where the first of them is a quarter behind (they differ by up to 17 %),
     // those with one where another number is a fifth ahead (they differ by up to
     // 15 %). Over 220 boxes of 12^3 to 129^3 the shape chosen is the best by hand
@@ -463,7 +464,7 @@ rt3d_status fs_tune(rt3d_grid *g, FsParams p) {
     int pick = 0;
     for (int i : order) {
         const int c = i < 0 ? 0 : i, per = kFsShapes[c].rays_per_thread;
-        const bool longer = i > 0 && t[0] > 0.2f;
+        const bool longer = i > 0 && best > 0.2f;
         // above 2^25 voxels, or where memory is short, the four-characteristic kernel's
         // 96 bytes a voxel are left to the solver's vectors
         if ((longer && per == 1 && best_many < 0.8f * t[0]) ||

@@ -1,6 +1,7 @@
 """Device memory that formal solutions can do without (the four-characteristic
 kernels' buffers: 96 bytes a voxel, 224 more with Lambda*): held only while the
-grid's shape or its Lambda* uses them, and not taken where memory is short."""
+grid's shape or its Lambda* uses them (from 16 MB on), and not taken where memory
+is short."""
 import numpy as np
 import pytest
 
@@ -19,17 +20,18 @@ def _problem(n, angles):
     return g, (d(chi), d(B), {"I_top": 0.3, "I_bottom": d(bc["I_bottom"])})
 
 
-@pytest.mark.parametrize("n", [(12, 10, 9), (33, 33, 33)])
+@pytest.mark.parametrize("n", [(12, 10, 9), (57, 56, 57)])  # the last: 17 MB
 def test_kept_while_in_use(n):
     g, args = _problem(n, (8, 16))
     N, base = n[0] * n[1] * n[2], g.info()["device_bytes"]
+    small = 96 * N < 1 << 24
     J = g.formal_solution(*args)  # tunes the shape
     info = g.info()
-    assert info["device_bytes"] - base == (96 * N if info["fs_shape"][1] == 4 else 0)
+    assert info["device_bytes"] - base == (96 * N if small or info["fs_shape"][1] == 4 else 0)
     for shape in [(64, 4, 1, 1), (128, 1, 1, 1), (64, 4, 1, 1), (128, 2, 1, 1)]:
         g.set_fs_shape(shape)
         assert ((g.formal_solution(*args) - J).abs() / J).max() < 2e-6, shape
-        assert g.info()["device_bytes"] - base == (96 * N if shape[1] == 4 else 0), shape
+        assert g.info()["device_bytes"] - base == (96 * N if small or shape[1] == 4 else 0), shape
     g.close()
 
 

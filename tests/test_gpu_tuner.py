@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,angles,ones,fours", [
-    ((20, 18, 12), (4, 8), 4, 3), ((97, 65, 65), (16, 32), 1, 3), ((65, 65, 129), (4, 16), 4, 1)])
+    ((20, 18, 12), (4, 8), 4, 3), ((129, 97, 65), (16, 32), 1, 3), ((16, 43, 113), (8, 16), 4, 1)])
 def test_candidates(n, angles, ones, fours):
     from paper_2102_01734_gb300 import rt3d
 
@@ -21,8 +21,8 @@ def test_candidates(n, angles, ones, fours):
     shapes = [rt3d.fs_tune_shape(i) for i in range(rt3d.FS_TUNE_SHAPES)]
     timed = {s: t for s, t in zip(shapes, info["fs_tune_ms"]) if t > 0}
     assert timed[info["fs_shape"]] == min(timed.values()) and shapes[0] in timed
-    # a 65 x 65 x 129 box with 64 angles takes some 0.4 ms, with four characteristics
-    # a thread a third longer; on the 97 x 65 x 65 one these are a quarter ahead
+    # the narrow box takes some 0.27 ms, with four characteristics a thread twice as
+    # long; on the wide one these are 30 % ahead
     assert [sum(s[1] == k for s in timed) for k in (1, 2, 4)] == [ones, 1, fours]
     g.set_fs_shape(shapes[1])
     other = g.formal_solution(d(chi), d(B), {"I_bottom": d(bc["I_bottom"])})
